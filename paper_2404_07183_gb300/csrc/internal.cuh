@@ -82,6 +82,24 @@ __device__ __forceinline__ bool block_sees_error(const Header* h)
     return __syncthreads_or(threadIdx.x == 0 && h->err != kNoError) != 0;
 }
 
+// Line m of the upper triangle of an N x N matrix that holds entry t, where
+// line m has N - m entries and starts at m N - m (m - 1) / 2: with R entries
+// from t to the end, L = N - m is the smallest L with L (L + 1) / 2 >= R.  A
+// float32 square root places it to within a few lines and integers make it
+// exact.  (A float64 square root costs 20 and more float64 operations, each
+// 65-77 issue cycles of its sub-partition on GB300.)
+__device__ __forceinline__ int64_t upper_line(int64_t N, int64_t t)
+{
+    const int64_t R = N * (N + 1) / 2 - t;
+    const float r = (float)(uint32_t)((uint64_t)R >> 32) * 4294967296.0f + (float)(uint32_t)R;
+    int64_t L = (int64_t)(uint32_t)sqrtf(r + r);
+    if (L > N) L = N;
+    if (L < 1) L = 1;
+    while (L > 1 && (L - 1) * L / 2 >= R) --L;
+    while (L * (L + 1) / 2 < R) ++L;
+    return N - L;
+}
+
 // Tile t of the queue (longest PCFs first) -> (row block bi, column block bj).
 // Symmetric (bi <= bj, NB blocks): line m of the triangle holds NB - m tiles
 // and starts at tile m NB - m (m - 1) / 2.  Order 1: line m is row block m,
@@ -93,12 +111,7 @@ __device__ __forceinline__ void decode_upper_tile(int64_t NB, int64_t t, int ord
                                                   int64_t& bi, int64_t& bj)
 {
     auto start = [NB](int64_t m) { return m * NB - m * (m - 1) / 2; };
-    const double q = 2.0 * (double)NB + 1.0;
-    const double disc = q * q - 8.0 * (double)t;
-    int64_t m = (int64_t)((q - sqrt(disc > 0.0 ? disc : 0.0)) * 0.5);
-    if (m < 0) m = 0;
-    while (m > 0 && start(m) > t) --m;
-    while (start(m + 1) <= t) ++m;
+    const int64_t m = upper_line(NB, t);
     if (order) {
         bi = m;
         bj = NB - 1 - (t - start(m));

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256, 4) mergepath_kernel(const WalkArgs a, int
                 const T h = (MI == MI_GRAM) ? lfv * lgv : fabs(lfv - lgv);
                 double Iv = I[m];
                 if (h != T(0)) Iv = (h > T(0)) ? (double)INFINITY : -(double)INFINITY;
-                const double Fv = finalize_root(a.metric[m], a.root[m], a.p[m], Iv);
+                const double Fv = finalize_root_rt(a.metric[m], a.root[m], a.p[m], Iv);
                 void* out = a.out[m];
                 auto put = [&](int64_t idx) {
                     if (a.out_f64) reinterpret_cast<double*>(out)[idx] = Fv;

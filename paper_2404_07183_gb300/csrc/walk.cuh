@@ -47,6 +47,7 @@
 #pragma once
 
 #include <cmath>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -112,6 +113,7 @@ template <> struct Acc<kF32> {
     __device__ __forceinline__ void add(float h, float dt) { s = fmaf(h, dt, s); }
     __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value() const { return (double)s; }
+    __device__ __forceinline__ void pair(float& hi, float& lo) const { hi = s; lo = 0.f; }
 };
 // Kahan's compensated summation, one rectangle term per add.  The term
 // h * dt is formed inside the fused multiply-add that also removes the
@@ -130,6 +132,12 @@ template <> struct Acc<kF32C> {
     }
     __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+    // the sum s - c as float32 hi + lo (exact for |s| >= |c|)
+    __device__ __forceinline__ void pair(float& hi, float& lo) const
+    {
+        hi = __fsub_rn(s, c);
+        lo = __fsub_rn(__fsub_rn(s, hi), c);
+    }
 };
 
 // Block-compensated float32: the rectangle terms are summed by FMA into a
@@ -151,6 +159,12 @@ template <> struct Acc<kF32B> {
         part = 0.f;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+    // the sum s - c as float32 hi + lo (exact for |s| >= |c|)
+    __device__ __forceinline__ void pair(float& hi, float& lo) const
+    {
+        hi = __fsub_rn(s, c);
+        lo = __fsub_rn(__fsub_rn(s, hi), c);
+    }
 };
 
 template <int COMBO, int PREC, typename T>
@@ -281,13 +295,75 @@ __device__ __forceinline__ double first_end(double a, double b)
     return __double_as_longlong(a) <= __double_as_longlong(b) ? a : b;
 }
 
-__device__ __forceinline__ double finalize_root(int metric, int root, double p, double I)
+// r(I) of one metric (its exponent is known at compile time but for MI_LP).
+template <int MI>
+__device__ __forceinline__ double finalize_root(int root, double p, double I)
+{
+    if (MI == MI_L1 || MI == MI_GRAM || !root) return I;
+    if (MI == MI_L2) return sqrt(I);
+    return pow(I, 1.0 / (MI == MI_L3 ? 3.0 : p));
+}
+
+// The same with the exponent taken from the request.
+__device__ __forceinline__ double finalize_root_rt(int metric, int root, double p, double I)
 {
     if (!root || metric == PCF_GRAM) return I;
     double e = metric == PCF_L1 ? 1.0 : metric == PCF_L2 ? 2.0 : p;
     if (e == 1.0) return I;
     if (e == 2.0) return sqrt(I);
     return pow(I, 1.0 / e);
+}
+
+// r(hi + lo) of a float32 walk rounded to float32, without float64 arithmetic
+// where a float32 root and one correction step do: with x = hi and r close to
+// its root, r^2 and r^3 are formed with their rounding errors (fma), so the
+// correction (x + lo - r^p) / (p r^(p-1)) is good to about 2^-22 of itself and
+// r plus it to about 2^-44 before the one rounding to float32.  (On GB300 a
+// float64 operation or conversion occupies a sub-partition for 65-77 cycles:
+// the float64 square root and roundings of a pair cost as much as 50 of its
+// merge steps, and pow several hundred.)
+template <int MI>
+__device__ __forceinline__ float finalize_root_f32(int root, double p, float hi, float lo)
+{
+    if (MI == MI_L1 || MI == MI_GRAM || !root) return hi;
+    if constexpr (MI == MI_L2 || MI == MI_L3) {
+        if (hi == 0.f && lo == 0.f) return 0.f;
+        if (hi > 0x1p-80f && hi < 0x1p126f) {      // residuals stay normal
+            if constexpr (MI == MI_L2) {
+                const float r = __fsqrt_rn(hi);
+                const float t = __fadd_rn(__fmaf_rn(-r, r, hi), lo);
+                return __fadd_rn(r, __fdividef(t, r + r));
+            } else {
+                const float r = cbrtf(hi);
+                const float q = __fmul_rn(r, r), qe = __fmaf_rn(r, r, -q);
+                const float c = __fmul_rn(q, r);
+                const float ce = __fmaf_rn(qe, r, __fmaf_rn(q, r, -c));   // r^3 = c + ce
+                const float t = __fadd_rn(__fsub_rn(__fsub_rn(hi, c), ce), lo);
+                return __fadd_rn(r, __fdividef(t, 3.f * q));
+            }
+        }
+    }
+    return (float)finalize_root<MI>(root, p, (double)hi + (double)lo);
+}
+
+// x != 0 and x != y without the float64 pipe (finite values).
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.f; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool differ(float x, float y) { return x != y; }
+__device__ __forceinline__ bool differ(double x, double y)
+{
+    return __double_as_longlong(x) != __double_as_longlong(y) && (nonzero(x) || nonzero(y));
+}
+
+// Sign of h on the last intervals [t_last, inf) of a pair: 0 when it adds
+// nothing, else the integral is that sign times inf.
+template <int MI, typename T>
+__device__ __forceinline__ int tail_sign(T vf, T vg)
+{
+    if (MI != MI_GRAM) return differ(vf, vg) ? 1 : 0;
+    if (!nonzero(vf) || !nonzero(vg)) return 0;
+    const T h = vf * vg;                       // may underflow to 0
+    return h > T(0) ? 1 : h < T(0) ? -1 : 0;
 }
 
 // Integral of the weight over a rectangle [l, l + dt): dt itself (WEIGHT 0),
@@ -365,7 +441,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     // window end per split candidate: [0] rows' minimum, [1] columns'
     __shared__ K sT1part[2][kSplits];
     __shared__ int sSplit;                          // split of the staged windows
-    __shared__ int64_t sTile;
+    __shared__ int64_t sUnit;
+    __shared__ int64_t sBlock[CTAS < 3 ? 2 : 1];    // the unit's row and column block
 
     if (gated_off(a.gate, a.gate_want64)) return;   // the other walk of an AUTO64 call
     if (block_sees_error(a.hdr)) return;
@@ -423,18 +500,35 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     const unsigned even_base_f = (unsigned)(pf >> 4) * regionBytes + (unsigned)(pf & 15) * sizeof(E);
     const unsigned even_base_g = (unsigned)(pg >> 4) * regionBytes + (unsigned)(pg & 15) * sizeof(E);
 
+    // Work units.  Thread 0 takes the next ticket while this unit is walked
+    // and decodes a unit for the CTA (decoded by every thread, a unit cost the
+    // CTA about 400 warp instructions and an atomic's latency).  The three-CTA
+    // schedules have no register for the ticket in flight: every thread
+    // decodes there.
+    constexpr bool kLean = CTAS < 3;
+    unsigned long long ticket = 0;
+    if (kLean && tid == 0) ticket = atomicAdd(&a.hdr->tiles, 1ull);
     for (;;) {
         if (tid == 0) {
-            const int64_t k = (int64_t)atomicAdd(&a.hdr->tiles, 1ull);
-            sTile = (a.shard_index + (k / UNITS) * a.shard_count) * UNITS + (k % UNITS);
+            const int64_t k = (int64_t)(kLean ? ticket : atomicAdd(&a.hdr->tiles, 1ull));
+            const int64_t u = (a.shard_index + (k / UNITS) * a.shard_count) * UNITS + (k % UNITS);
+            sUnit = u;
+            if (kLean && u / UNITS < a.ntiles) {
+                int64_t r, c;
+                decode_tile(a, u / UNITS, r, c);
+                sBlock[0] = r;
+                sBlock[1] = c;
+                ticket = atomicAdd(&a.hdr->tiles, 1ull);
+            }
         }
         __syncthreads();
-        const int64_t unit = sTile;
+        const int64_t unit = sUnit;
         const int64_t t = unit / UNITS;
         if (t >= a.ntiles) break;
         const int half = (int)(unit - t * UNITS);
         int64_t bi, bj;
-        decode_tile(a, t, bi, bj);
+        if constexpr (kLean) { bi = sBlock[0]; bj = sBlock[1]; }
+        else decode_tile(a, t, bi, bj);
         const int64_t col0 = bj * kTile + half * TCOLS;   // first column of this unit
 
         // unit metadata
@@ -715,33 +809,80 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
                     smem + (kAdapt ? slot_base(pg, wr_last, wc_last) : even_base_g) +
                     (unsigned)(sLen[pg] - 1 - sS[pg]) * kRow));
             }
-#pragma unroll
-            for (int m = 0; m < NM; ++m) {
-                const int MI = combo_metric(COMBO, m);
-                double I = acc.value(m);
-                const T h = (MI == MI_GRAM) ? vlf * vlg : fabs(vlf - vlg);
-                if (!bounded && h != T(0)) I = (h > T(0)) ? (double)INFINITY : -(double)INFINITY;
-                const double F = finalize_root(a.metric[m], a.root[m], a.p[m], I);
-                void* out = a.out[m];
-                auto put = [&](int64_t idx) {
-                    if (a.out_f64) reinterpret_cast<double*>(out)[idx] = F;
-                    else reinterpret_cast<float*>(out)[idx] = (float)F;
+            if constexpr (kLean) {
+                auto store = [&](auto m_c) {
+                    constexpr int m = decltype(m_c)::value;
+                    constexpr int MI = combo_metric(COMBO, m);
+                    const int sgn = bounded ? 0 : tail_sign<MI>(vlf, vlg);
+                    double F = 0.0;
+                    float Ff = 0.f;
+                    bool f64 = true;
+                    if constexpr (sizeof(T) == 4) f64 = a.out_f64 != 0;
+                    if (f64) {
+                        double I = acc.value(m);
+                        if (sgn) I = sgn > 0 ? (double)INFINITY : -(double)INFINITY;
+                        F = finalize_root<MI>(a.root[m], a.p[m], I);
+                        if (!a.out_f64) Ff = (float)F;
+                    } else if constexpr (sizeof(T) == 4) {
+                        float hi, lo;
+                        acc.a[m].pair(hi, lo);
+                        if (sgn) Ff = sgn > 0 ? INFINITY : -INFINITY;   // r(inf) = inf
+                        else Ff = finalize_root_f32<MI>(a.root[m], a.p[m], hi, lo);
+                    }
+                    void* out = a.out[m];
+                    auto put = [&](int64_t idx) {
+                        if (a.out_f64) reinterpret_cast<double*>(out)[idx] = F;
+                        else reinterpret_cast<float*>(out)[idx] = Ff;
+                    };
+                    if (!a.symmetric) {
+                        put(i * a.ld_out + j);
+                    } else if (a.layout == PCF_OUT_FULL) {
+                        put(i * a.ld_out + j);
+                        if (bi != bj) put(j * a.ld_out + i);
+                    } else if (a.layout == kOutRowsInputColsSorted) {
+                        put(i * a.ld_out + gj);
+                        if (bi != bj) put(j * a.ld_out + gi);
+                    } else if (a.layout == PCF_OUT_FULL_SORTED) {
+                        put(gi * a.ld_out + gj);
+                        if (bi != bj) put(gj * a.ld_out + gi);
+                    } else {
+                        const int64_t N = a.ld_out;
+                        const int64_t lo2 = i < j ? i : j, hi2 = i < j ? j : i;
+                        if (bi != bj || i <= j) put(lo2 * N - lo2 * (lo2 - 1) / 2 + (hi2 - lo2));
+                    }
                 };
-                if (!a.symmetric) {
-                    put(i * a.ld_out + j);
-                } else if (a.layout == PCF_OUT_FULL) {
-                    put(i * a.ld_out + j);
-                    if (bi != bj) put(j * a.ld_out + i);
-                } else if (a.layout == kOutRowsInputColsSorted) {
-                    put(i * a.ld_out + gj);
-                    if (bi != bj) put(j * a.ld_out + gi);
-                } else if (a.layout == PCF_OUT_FULL_SORTED) {
-                    put(gi * a.ld_out + gj);
-                    if (bi != bj) put(gj * a.ld_out + gi);
-                } else {
-                    const int64_t N = a.ld_out;
-                    const int64_t lo2 = i < j ? i : j, hi2 = i < j ? j : i;
-                    if (bi != bj || i <= j) put(lo2 * N - lo2 * (lo2 - 1) / 2 + (hi2 - lo2));
+                store(std::integral_constant<int, 0>{});
+                if constexpr (NM > 1) store(std::integral_constant<int, 1>{});
+                if constexpr (NM > 2) store(std::integral_constant<int, 2>{});
+            } else {
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    const int MI = combo_metric(COMBO, m);
+                    double I = acc.value(m);
+                    const T h = (MI == MI_GRAM) ? vlf * vlg : fabs(vlf - vlg);
+                    if (!bounded && h != T(0)) I = (h > T(0)) ? (double)INFINITY : -(double)INFINITY;
+                    const double F = finalize_root_rt(a.metric[m], a.root[m], a.p[m], I);
+                    void* out = a.out[m];
+                    auto put = [&](int64_t idx) {
+                        if (a.out_f64) reinterpret_cast<double*>(out)[idx] = F;
+                        else reinterpret_cast<float*>(out)[idx] = (float)F;
+                    };
+                    if (!a.symmetric) {
+                        put(i * a.ld_out + j);
+                    } else if (a.layout == PCF_OUT_FULL) {
+                        put(i * a.ld_out + j);
+                        if (bi != bj) put(j * a.ld_out + i);
+                    } else if (a.layout == kOutRowsInputColsSorted) {
+                        put(i * a.ld_out + gj);
+                        if (bi != bj) put(j * a.ld_out + gi);
+                    } else if (a.layout == PCF_OUT_FULL_SORTED) {
+                        put(gi * a.ld_out + gj);
+                        if (bi != bj) put(gj * a.ld_out + gi);
+                    } else {
+                        const int64_t N = a.ld_out;
+                        const int64_t lo2 = i < j ? i : j, hi2 = i < j ? j : i;
+                        if (bi != bj || i <= j) put(lo2 * N - lo2 * (lo2 - 1) / 2 + (hi2 - lo2));
+                    }
                 }
             }
         }
