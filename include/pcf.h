@@ -156,10 +156,11 @@ enum pcf_cross_flags {
  *   PCF_SCHED_TILE_512X3  32 x 16 half tiles, three 512-thread CTAs per SM
  *                         (at most 40 registers per thread, a third of the
  *                         shared memory each)
- *   PCF_SCHED_MERGEPATH   one warp per pair, the pair's merge split across
- *                         the 32 lanes (for few, long pairs)
- *   PCF_SCHED_AUTO        merge path when there are fewer tiles than half the
- *                         SMs, else TILE_1024 */
+ *   PCF_SCHED_MERGEPATH   one pair per warp, CTA or cluster of CTAs (by its
+ *                         length), the pair's merge split across the threads
+ *                         (for few pairs)
+ *   PCF_SCHED_AUTO        merge path for few pairs (14,000 for float32 walks,
+ *                         45,000 for float64), else TILE_1024 */
 enum pcf_sched_kernel {
     PCF_SCHED_AUTO = 0, PCF_SCHED_TILE_1024 = 1, PCF_SCHED_TILE_512X2 = 2,
     PCF_SCHED_MERGEPATH = 3, PCF_SCHED_TILE_512X3 = 4

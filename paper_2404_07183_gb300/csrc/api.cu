@@ -410,11 +410,47 @@ int check_window(const pcf_window* w)
     return PCF_OK;
 }
 
-// kernel_out: the schedule kernel the call resolves to (AUTO decided here).
-// unit0: first work unit (tile schedules; the launch ends at wa.ntiles).
-int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int form,
+// Pairs up to which PCF_SCHED_AUTO takes the merge path.  It works in
+// proportion to the pairs, while a tile walk of few tiles takes one unit's
+// time however few pairs there are.  Measured (ms, tiles / merge path):
+// float32 walks, 5,050 pairs of 2 x 450 points 0.076 / 0.058 and of 2 x 900
+// 0.111 / 0.060, 20,100 pairs of 2 x 1,350 0.160 / 0.233 and of 2 x 275 (three
+// metrics) 0.109 / 0.100; float64 walks, 20,100 pairs of 2 x 55 points 0.109 /
+// 0.058 and of 2 x 275 (three metrics) 1.10 / 0.22, 45,150 pairs of 2 x 55
+// 0.109 / 0.100 and of 2 x 540 0.62 / 0.68.
+constexpr int64_t kMpPairsF32 = 14000, kMpPairsF64 = 45000;
+
+int auto_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool round,
+                bool windowed, bool weighted, const pcf_schedule* sched)
+{
+    const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
+    if (!windowed && pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32))
+        return PCF_SCHED_MERGEPATH;
+    return PCF_SCHED_TILE_1024;
+}
+
+bool is_windowed(const pcf_window* w)
+{
+    return w && (w->a > 0.0 || !std::isinf(w->b) || w->lambda > 0.0);
+}
+
+// Whether FULL matrices are written with sorted columns and put back in place
+// by a second pass (whole DRAM sectors from the walk).  Not when the rows do
+// not fit that pass, nor for a shard, nor for small matrices, whose scattered
+// entries cost less than the two launches (97 x 97 float64: 97 -> 79 us per call;
+// three 701 x 701 float32 matrices, 5.9 MB: 15 us slower written directly).
+constexpr int64_t kDirectFullBytes = 2ll << 20;
+
+bool full_in_two_passes(const WalkArgs& wa, int nF, int layout, const pcf_schedule* sched)
+{
+    return layout == PCF_OUT_FULL && !(sched && sched->shard_count > 1) &&
+           permute_cols_fits(wa.ld_out, wa.out_f64) &&
+           wa.ld_out * wa.ld_out * (wa.out_f64 ? 8 : 4) * nF > kDirectFullBytes;
+}
+
+int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int form, bool round,
               const pcf_schedule* sched, const pcf_window* win, cudaStream_t s,
-              int64_t unit0 = 0, int* kernel_out = nullptr)
+              int64_t unit0 = 0)
 {
     const int elem_bytes = pack_elem_bytes(form);
     const bool keyed = form == kPackKeyed;
@@ -422,16 +458,15 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
     wa.lo = win ? win->a : 0.0;
     wa.hi = win ? win->b : (double)INFINITY;
     wa.lambda = win ? win->lambda : 0.0;
-    const bool windowed = wa.lo > 0.0 || !std::isinf(wa.hi) || wa.lambda > 0.0;
+    const bool windowed = is_windowed(win);
     const bool weighted = wa.lambda > 0.0;
     wa.shard_count = (sched && sched->shard_count > 1) ? sched->shard_count : 1;
     wa.shard_index = (sched && sched->shard_count > 1) ? sched->shard_index : 0;
     int kernel = sched ? sched->kernel : PCF_SCHED_AUTO;
     if (kernel == PCF_SCHED_AUTO)
-        kernel = (wa.ntiles * 2 < sms && !windowed) ? PCF_SCHED_MERGEPATH : PCF_SCHED_TILE_1024;
+        kernel = auto_kernel(wa, F, nF, form, round, windowed, weighted, sched);
     if (windowed && kernel == PCF_SCHED_MERGEPATH) return PCF_EUNSUPPORTED;
     if (weighted && kernel != PCF_SCHED_TILE_1024) return PCF_EUNSUPPORTED;
-    if (kernel_out) *kernel_out = kernel;
     if (kernel == PCF_SCHED_MERGEPATH && unit0 != 0) return PCF_EINVAL;
 
     int64_t grid = 0;
@@ -439,10 +474,6 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
     int64_t npairs = 0;
     if (kernel == PCF_SCHED_MERGEPATH) {
         npairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
-        grid = (int64_t)sms * 4;
-        const int64_t need = (npairs + 7) / 8;    // 8 warps per block
-        if (grid > need) grid = need;
-        if (grid < 1) return PCF_OK;
     } else {
         const bool half = kernel == PCF_SCHED_TILE_512X2 || kernel == PCF_SCHED_TILE_512X3;
         const int ctas = kernel == PCF_SCHED_TILE_512X3 ? 3 : (half ? 2 : 1);
@@ -474,7 +505,8 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
             wa.root[k] = f.apply_root ? 1 : 0;
             wa.p[k] = f.metric == PCF_LP ? f.p : (f.metric == PCF_L2 ? 2.0 : 1.0);
         }
-        reset_tiles_kernel<<<1, 1, 0, s>>>(wa.hdr, (unsigned long long)unit0);
+        if (kernel != PCF_SCHED_MERGEPATH)
+            reset_tiles_kernel<<<1, 1, 0, s>>>(wa.hdr, (unsigned long long)unit0);
         cudaError_t e;
         const int g = (int)grid;
         // launcher of (schedule, precision, form)
@@ -488,7 +520,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
                     : precision == PCF_PREC_F32_COMP ? (keyed ? launch_mergepath_f32ck : launch_mergepath_f32c)
                     : precision == PCF_PREC_F32_BLOCK ? (keyed ? launch_mergepath_f32bk : launch_mergepath_f32b)
                     : (keyed ? launch_mergepath_f32k : launch_mergepath_f32);
-            e = mp(L.combo, wa, npairs, g, s);
+            e = mp(L.combo, wa, npairs, wa.mean_steps, s);
         } else if (kernel == PCF_SCHED_TILE_512X3) {
             e = PCF_PICK(t512x3)(L.combo, wa, g, smem, s);
         } else if (kernel == PCF_SCHED_TILE_512X2) {
@@ -513,16 +545,16 @@ int run_walks_for(WalkArgs& wa, const pcf_integral* F, int nF, const Prec& pr, i
 {
     if (!pr.auto64 || form == kPackF64) {
         wa.gate = nullptr;
-        return run_walks(wa, F, nF, pr.base, form, sched, win, s, unit0);
+        return run_walks(wa, F, nF, pr.base, form, pr.round, sched, win, s, unit0);
     }
     wa.gate = &wa.hdr->need64;
     wa.gate_want64 = 0;
-    int rc = run_walks(wa, F, nF, pr.base, form, sched, win, s, unit0);
+    int rc = run_walks(wa, F, nF, pr.base, form, pr.round, sched, win, s, unit0);
     if (rc != PCF_OK) return rc;
     WalkArgs w64 = wa;
     w64.gate_want64 = 1;
     w64.bound_keys = nullptr;
-    return run_walks(w64, F, nF, PCF_PREC_F64, kPackF64, sched, win, s, unit0);
+    return run_walks(w64, F, nF, PCF_PREC_F64, kPackF64, false, sched, win, s, unit0);
 }
 
 // Bands of the symmetric tile order for streaming a matrix to the host.  The
@@ -715,15 +747,13 @@ int pcf_pairwise_ex(const pcf_csr* x, const pcf_integral* F, int nF, int precisi
     wa.perm_r = wa.perm_c = sv.perm;
     wa.n_r = wa.n_c = x->n;
     wa.nb_r = wa.nb_c = (x->n + kTile - 1) / kTile;
+    wa.mean_steps = 2 * (x->nnz / x->n);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;
     wa.out_f64 = out_dtype == PCF_F64;
     wa.ld_out = x->n;
-    // FULL matrices of one call (not a shard) whose rows fit the permutation
-    // pass: written with sorted columns, then put back in place
-    const bool cols_sorted = layout == PCF_OUT_FULL && !(schedule && schedule->shard_count > 1) &&
-                             permute_cols_fits(x->n, wa.out_f64);
+    const bool cols_sorted = full_in_two_passes(wa, nF, layout, schedule);
     wa.layout = cols_sorted ? kOutRowsInputColsSorted : layout;
     KElem* kp = reinterpret_cast<KElem*>(sv.packed);
     keyed_bounds(wa, window, form, ks, kp, kp, hdr, stream);
@@ -781,6 +811,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     wa.perm_r = wa.perm_c = sv.perm;
     wa.n_r = wa.n_c = N;
     wa.nb_r = wa.nb_c = (N + kTile - 1) / kTile;
+    wa.mean_steps = 2 * (x->nnz / N);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;
@@ -843,7 +874,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     memset(&sch, 0, sizeof sch);
     if (schedule) sch = *schedule;
     if (sch.kernel == PCF_SCHED_AUTO)
-        sch.kernel = wa.ntiles * 2 < sms ? PCF_SCHED_MERGEPATH : PCF_SCHED_TILE_1024;
+        sch.kernel = auto_kernel(wa, F, nF, form, pr.round, false, false, schedule);
     // `stream` continues after the last copy enqueued, also when a later
     // step fails (the caller may reuse the buffers after an error)
     auto join = [&]() -> bool {
@@ -991,6 +1022,7 @@ static int cross_impl(const pcf_csr* a, const pcf_csr* b, int64_t row_begin, int
     wa.nb_r = (rows + kTile - 1) / kTile;
     wa.nb_c = (b->n + kTile - 1) / kTile;
     wa.ntiles = wa.nb_r * wa.nb_c;
+    wa.mean_steps = a->nnz / (a->n > 0 ? a->n : 1) + b->nnz / b->n;   // (a: of the whole set)
     wa.symmetric = 0;
     wa.hdr = hdr;
     wa.layout = PCF_OUT_FULL;
@@ -1259,13 +1291,13 @@ int pcf_pairwise_weighted(const pcf_csr* x, const pcf_csr* w, const pcf_integral
     wa.perm_r = wa.perm_c = sv.perm;
     wa.n_r = wa.n_c = m.n;
     wa.nb_r = wa.nb_c = (m.n + kTile - 1) / kTile;
+    wa.mean_steps = 2 * (m.nnz / m.n);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;
     wa.out_f64 = out_dtype == PCF_F64;
     wa.ld_out = m.n;
-    const bool cols_sorted = layout == PCF_OUT_FULL && !(schedule && schedule->shard_count > 1) &&
-                             permute_cols_fits(m.n, wa.out_f64);
+    const bool cols_sorted = full_in_two_passes(wa, nF, layout, schedule);
     wa.layout = cols_sorted ? kOutRowsInputColsSorted : layout;
     KElem* kp = reinterpret_cast<KElem*>(sv.packed);
     keyed_bounds(wa, nullptr, form, ks, kp, kp, hdr, stream);

@@ -254,6 +254,7 @@ struct WalkArgs {
     int64_t n_r, n_c;
     int64_t nb_r, nb_c;      // tile blocks
     int64_t ntiles;
+    int64_t mean_steps;      // mean breakpoints of a pair (both PCFs), for the host's choices
     int symmetric;           // pairwise: upper-triangle tiles, R == C
     int tile_order;          // symmetric tile order: 0 = column blocks from the last
                              // down, 1 = row blocks from the first up (each with its
@@ -302,13 +303,14 @@ enum Combo : int {
 };
 
 // Launch the persistent tile walk for one precision, CTA size and metric
-// combination, or the warp-per-pair merge-path walk over `npairs` pairs.
+// combination, or the cooperative merge-path walk over `npairs` pairs of
+// `mean_steps` breakpoints (both PCFs) on average.
 #define PCF_DECL_WALK(name)                                                                     \
     cudaError_t launch_walk_##name##_t1024(int, const WalkArgs&, int, size_t, cudaStream_t);    \
     cudaError_t launch_walk_##name##_t512(int, const WalkArgs&, int, size_t, cudaStream_t);     \
     cudaError_t launch_walk_##name##_t512x3(int, const WalkArgs&, int, size_t, cudaStream_t);   \
     cudaError_t launch_walk_##name##_t1024w(int, const WalkArgs&, int, size_t, cudaStream_t);   \
-    cudaError_t launch_mergepath_##name(int, const WalkArgs&, int64_t, int, cudaStream_t);
+    cudaError_t launch_mergepath_##name(int, const WalkArgs&, int64_t, int64_t, cudaStream_t);
 PCF_DECL_WALK(f64)
 PCF_DECL_WALK(f32c)
 PCF_DECL_WALK(f32)

@@ -1,9 +1,9 @@
-// mergepath_f32ck.cu -- keyed warp-per-pair merge-path instantiations (float64 input), F32C precision.
+// mergepath_f32ck.cu -- keyed cooperative merge-path instantiations (float64 input), F32C precision.
 #include "mergepath.cuh"
 
 namespace pcfgb {
-cudaError_t launch_mergepath_f32ck(int combo, const WalkArgs& a, int64_t npairs, int grid, cudaStream_t s)
+cudaError_t launch_mergepath_f32ck(int combo, const WalkArgs& a, int64_t npairs, int64_t mean_steps, cudaStream_t s)
 {
-    return launch_mergepath_t<float, kF32C, true>(combo, a, npairs, grid, s);
+    return launch_mergepath_t<float, kF32C, true>(combo, a, npairs, mean_steps, s);
 }
 }  // namespace pcfgb

@@ -1,0 +1,65 @@
+"""The cooperative merge path at the edges of its slabs, groups and parts
+(needs a GPU).  A warp takes 256 advances per slab, a CTA 2,048; a pair goes to
+CTAs above 1,024 breakpoints on average and to clusters of 2, 4 or 8 CTAs above
+8,192, 16,384 and 32,768."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2404_07183_gb300 import synth
+
+from conftest import gpu_available, max_rel_error
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"f64": 1e-12, "f32c": 1e-5, "f32b": 1e-5}
+LENGTHS = [[1, 1, 2], [128, 129, 130, 1], [300, 213, 43, 600], [1025, 1024, 1023, 3],
+           [2049, 2048, 4100, 1], [4097, 4096, 5000], [9001, 8192, 7000], [16385, 20000, 12001]]
+
+
+@pytest.fixture(scope="module")
+def pcf():
+    if not gpu_available():
+        pytest.skip("no CUDA device")
+    import paper_2404_07183_gb300 as P
+    P.build.build()
+    return P
+
+
+@pytest.mark.parametrize("lens", LENGTHS, ids=lambda v: str(max(v)))
+@pytest.mark.parametrize("prec,dtype", [("f64", np.float64), ("f32c", np.float64),
+                                        ("f32c", np.float32), ("f32b", np.float32)])
+def test_slab_edges(pcf, lens, prec, dtype):
+    import torch
+    rng = np.random.default_rng(sum(lens))
+    s = synth.from_lengths(lens, lambda r, m: r.exponential(1.0, m),
+                           lambda r, o: np.where(np.isin(np.arange(o[-1]), o[1:] - 1), 0.0,
+                                                 r.standard_normal(o[-1])), rng, dtype)
+    x = pcf.PcfTensors.from_numpy(s, "cuda")
+    s64 = synth.PcfSet(s.offsets, s.times.astype(np.float64), s.values.astype(np.float64))
+    diag = np.array([oracle.segment_sq(*s64.pcf(i)) for i in range(s64.n)])
+    got = pcf.pcf_pairwise(x, ["l1", "l2", "gram"], precision=prec, out_dtype=torch.float64,
+                           schedule="mergepath")
+    again = pcf.pcf_pairwise(x, ["l1", "l2", "gram"], precision=prec, out_dtype=torch.float64,
+                             schedule="mergepath")
+    for m, g, h in zip(("l1", "l2", "gram"), got, again):
+        assert max_rel_error(m, g.cpu().numpy(), oracle.matrix(s64, metric=m), diag) <= TOL[prec], m
+        assert torch.equal(g, h), m                     # fixed order: the same bits
+
+
+@pytest.mark.parametrize("lens", [[300, 213, 43, 600], [9001, 8192, 7000]], ids=str)
+def test_dyadic_bitwise(pcf, lens):
+    """Integer times with many shared breakpoints: every partial sum is exact."""
+    import torch
+    rng = np.random.default_rng(5)
+    s = synth.from_lengths(lens, lambda r, m: r.integers(1, 3, m).astype(np.float64),
+                           lambda r, o: np.where(np.isin(np.arange(o[-1]), o[1:] - 1), 0.0,
+                                                 r.integers(-6, 7, o[-1])), rng, np.float64)
+    x = pcf.PcfTensors.from_numpy(s, "cuda")
+    for prec in ("f64", "f32c"):
+        got = pcf.pcf_pairwise(x, ["l1", "gram"], precision=prec, out_dtype=torch.float64,
+                               schedule="mergepath")
+        for m, g in zip(("l1", "gram"), got):
+            if prec == "f32c" and max(lens) > 1000:
+                continue                                # sums beyond 2^24
+            np.testing.assert_array_equal(g.cpu().numpy(), oracle.matrix(s, metric=m))
