@@ -160,7 +160,10 @@ enum pcf_cross_flags {
  *                         length), the pair's merge split across the threads
  *                         (for few pairs)
  *   PCF_SCHED_AUTO        merge path for few pairs (14,000 for float32 walks,
- *                         45,000 for float64), else TILE_1024 */
+ *                         45,000 for float64), else TILE_512X3 for float32
+ *                         walks of float32 input with one metric but general
+ *                         p, TILE_512X2 for the others, and TILE_1024 for
+ *                         rounded times, an explicit window or lambda > 0 */
 enum pcf_sched_kernel {
     PCF_SCHED_AUTO = 0, PCF_SCHED_TILE_1024 = 1, PCF_SCHED_TILE_512X2 = 2,
     PCF_SCHED_MERGEPATH = 3, PCF_SCHED_TILE_512X3 = 4
@@ -185,7 +188,7 @@ typedef struct pcf_schedule {
  * integrated per rectangle through its antiderivative (the time-dependent
  * combinations of Sec. 2.1 and Sec. 3).  For float32 walks a, b and lambda
  * are rounded to float32.  With b < inf nothing diverges.  Tile schedules
- * only (PCF_SCHED_AUTO picks TILE_1024); lambda > 0 runs on TILE_1024. */
+ * only (PCF_SCHED_AUTO picks one); lambda > 0 runs on TILE_1024. */
 typedef struct pcf_window {
     double a;
     double b;

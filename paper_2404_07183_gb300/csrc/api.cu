@@ -410,6 +410,27 @@ int check_window(const pcf_window* w)
     return PCF_OK;
 }
 
+// PCF_SCHED_AUTO for tile walks.  Measured (GB300, walk alone, ms, one
+// 1024-thread CTA per SM / two / three 512-thread CTAs): stable-rank curves
+// N = 6,000, float64 input in float32 with one metric 9.99 / 9.42 / 9.52, with
+// three 11.57 / 10.62 / 11.00; float32 Gram of 30,000 log-normal curves
+// 96.3 / 82.0 / 76.9; float32 cross 3,001 x 4,000 of 1,000 points with three
+// metrics 20.8 / 19.2 / 19.8; float64 N = 1,000 0.461 / 0.407 / 0.414.  Two
+// CTAs let one issue while the other waits at a tile barrier.  The third pays
+// where 40 registers hold the walk: 8-byte elements and one metric without
+// pow.  TILE_1024 stays where its larger window decides what is accepted
+// (rounded times: coincident times must fit one window; an explicit window)
+// and for the exp(-lambda t) weights, which only it has.
+int auto_tile_kernel(const pcf_integral* F, int nF, int form, bool round, bool weighted,
+                     bool explicit_window)
+{
+    if (weighted || round || explicit_window) return PCF_SCHED_TILE_1024;
+    if (form != kPackF32) return PCF_SCHED_TILE_512X2;
+    for (const Launch& L : plan(F, nF))
+        if (L.n > 1 || L.combo == kComboLP) return PCF_SCHED_TILE_512X2;
+    return PCF_SCHED_TILE_512X3;
+}
+
 // Pairs up to which PCF_SCHED_AUTO takes the merge path.  It works in
 // proportion to the pairs, while a tile walk of few tiles takes one unit's
 // time however few pairs there are.  Measured (ms, tiles / merge path):
@@ -426,7 +447,7 @@ int auto_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, boo
     const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
     if (!windowed && pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32))
         return PCF_SCHED_MERGEPATH;
-    return PCF_SCHED_TILE_1024;
+    return auto_tile_kernel(F, nF, form, round, weighted, sched && sched->window != 0);
 }
 
 bool is_windowed(const pcf_window* w)
