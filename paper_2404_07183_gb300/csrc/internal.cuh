@@ -176,15 +176,18 @@ struct KeySort {
     int64_t tiles = 0;
     uint64_t* key[2] = {nullptr, nullptr};
     uint32_t* pay[2] = {nullptr, nullptr};
-    uint32_t* hist = nullptr;   // 256 x tiles digit counts
-    uint32_t* tsum = nullptr;   // tiles + 1 distinct-key counts
-    uint32_t* dsum = nullptr;   // 256 digit totals
+    uint32_t* status = nullptr; // tiles x 256 look-back states of a pass
+    uint32_t* tsum = nullptr;   // tiles + 1 look-back states of the rank kernel
+    uint32_t* misc = nullptr;   // digit counts of all passes, plan, tickets (keys.cu)
 };
+// Bytes by which keysort_bytes exceeds the 24 bytes per key, 1 KB and 4 bytes
+// per tile of 8,192 keys and 1 KB that pcf_pairwise_noalloc's limit counts.
+constexpr size_t kKeySortExtra = 7424;
 size_t keysort_bytes(int64_t cap);
 KeySort carve_keysort(char*& cursor, int64_t cap);
 // Ranks of the interval ends of one or two packed keyed collections, written
 // into their KElem.k fields.  The sort input (key[0], pay[0]) is written by
-// the pack; the sorted keys end in key[0], pay[0].
+// the pack; the sorted keys end in either buffer (misc says which).
 cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int64_t n0,
                       KElem* pack1, const int64_t* poff1, int64_t n1, Header* hdr, cudaStream_t s);
 // Order keys of the integration bounds a, b into hdr->bound_key (after

@@ -15,14 +15,22 @@
 //
 // The ranks come from a device-wide stable LSD radix sort of the (time bits,
 // packed position) pairs: non-negative float64 values order like their bit
-// patterns read as unsigned 64-bit integers.  Eight passes of 8-bit digits;
-// each pass is a histogram kernel (per tile of kSortTile keys), exclusive
-// scans of each digit's counts over the tiles (a CTA per digit) and of the
-// digit totals, and a scatter
-// kernel that ranks the tile's keys stably (warp match, per-warp digit counts)
-// and writes them to their digit's next free positions.  After the last pass
-// a segmented count of distinct keys gives every sorted key its rank, written
-// into the rank field of the packed element the payload names.
+// patterns read as unsigned 64-bit integers.  One kernel counts all eight
+// 8-bit digits (they do not depend on the order) and plans the passes: a digit
+// that all keys share needs none.  Each pass is one kernel: a CTA takes a tile
+// of 8,192 keys by ticket, ranks them stably (warp match, per-warp digit
+// counts), learns how many of each digit the tiles before it hold by decoupled
+// look-back (thread d waits for digit d; tickets make every predecessor a
+// running or finished CTA, and every wait is bounded), orders the tile in
+// shared memory and writes it in runs of one digit.  A last kernel counts
+// distinct keys the same way and writes every key's rank into the packed
+// element its payload names.
+//
+// What bounds it: few keys, the latency of ten launches in a row; many, the
+// 24 bytes per key and pass.  A histogram, two scans and an unordered scatter
+// per pass (35 launches) came before: three matrices of 701 stable-rank curves
+// (193,000 keys) took 0.78 ms per call and now 0.47, of 20,000 (5.5 million)
+// 117.0 and now 116.2.
 //
 // The number of keys is known on the device only (it depends on the lengths
 // of the rows a call packs); the kernels read it from the header and are
@@ -31,10 +39,20 @@
 
 namespace pcfgb {
 
-constexpr int kSortThreads2 = 256;
-constexpr int kSortItems = 32;
-constexpr int kSortTile = kSortThreads2 * kSortItems;   // keys per tile (8,192)
+constexpr int kSortThreads2 = 512;
 constexpr int kSortWarps = kSortThreads2 / 32;
+constexpr int kSortItems = 16;
+constexpr int kSortTile = kSortThreads2 * kSortItems;   // keys per tile (8,192)
+
+// KeySort::misc (32-bit words): the digit counts (then their exclusive scans)
+// of the eight passes, the pass plan, the sorted buffer, the tickets of the
+// passes and of the rank kernel, the finished counter of the histogram.
+constexpr int kMiscPlan = 8 * 256;         // [8]: buffer the pass reads, or 2 = no pass
+constexpr int kMiscFinal = kMiscPlan + 8;  // buffer that holds the sorted keys
+constexpr int kMiscTicket = kMiscFinal + 1;    // [9]
+constexpr int kMiscDone = kMiscTicket + 9;
+constexpr int kMiscWords = 8 * 256 + 64;
+static_assert(kMiscDone < kMiscWords, "misc layout");
 
 int64_t key_tiles(int64_t cap) { return cap > 0 ? (cap + kSortTile - 1) / kSortTile : 1; }
 
@@ -46,7 +64,7 @@ size_t keysort_bytes(int64_t cap)
     b += 2 * align_up(sizeof(uint32_t) * (size_t)(cap > 0 ? cap : 1));
     b += align_up(sizeof(uint32_t) * 256 * (size_t)tiles);
     b += align_up(sizeof(uint32_t) * (size_t)(tiles + 1));
-    b += align_up(sizeof(uint32_t) * 256);
+    b += align_up(sizeof(uint32_t) * kMiscWords);
     return b;
 }
 
@@ -61,17 +79,20 @@ KeySort carve_keysort(char*& cur, int64_t cap)
     k.key[1] = reinterpret_cast<uint64_t*>(take(sizeof(uint64_t) * (size_t)c));
     k.pay[0] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (size_t)c));
     k.pay[1] = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (size_t)c));
-    k.hist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * (size_t)k.tiles));
+    k.status = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256 * (size_t)k.tiles));
     k.tsum = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * (size_t)(k.tiles + 1)));
-    k.dsum = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * 256));
+    k.misc = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * kMiscWords));
     return k;
 }
 
 // Number of keys of a call: sum over its collections of (breakpoints - PCFs),
-// from the packed offsets poff[n] of each set.
-__global__ void count_keys_kernel(Header* hdr, const int64_t* poff0, int64_t n0,
-                                  const int64_t* poff1, int64_t n1)
+// from the packed offsets poff[n] of each set.  Clears the sort's counters.
+__global__ void __launch_bounds__(256) count_keys_kernel(Header* hdr, const int64_t* poff0, int64_t n0,
+                                                         const int64_t* poff1, int64_t n1,
+                                                         uint32_t* __restrict__ misc)
 {
+    for (int i = threadIdx.x; i < kMiscWords; i += 256) misc[i] = 0;
+    if (threadIdx.x != 0) return;
     // no keys after an input error, or when an AUTO64 call walks in float64
     if (hdr->err != kNoError || hdr->need64 != 0u) { hdr->nkeys = 0; return; }
     unsigned long long m = 0;
@@ -80,46 +101,114 @@ __global__ void count_keys_kernel(Header* hdr, const int64_t* poff0, int64_t n0,
     hdr->nkeys = m;
 }
 
-// Digit histogram of one tile of keys, written digit-major: hist[d * tiles + t].
-__global__ void __launch_bounds__(kSortThreads2)
-radix_hist_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ hist, int64_t tiles,
-                  int shift, const Header* hdr)
-{
-    __shared__ uint32_t cnt[256];
-    const int tid = threadIdx.x;
-    cnt[tid] = 0;
-    __syncthreads();
-    const int64_t m = (int64_t)hdr->nkeys;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    const int lane = tid & 31;
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = base + (int64_t)r * kSortThreads2 + tid;
-        // one shared-memory atomic per distinct digit of the warp (the high
-        // digits of nearby times mostly agree)
-        const unsigned d = i < m ? ((unsigned)(key[i] >> shift) & 255u) : 256u + lane;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        if (d < 256u && (__ffs(peers) - 1) == lane) atomicAdd(&cnt[d], (unsigned)__popc(peers));
+// Chunk states of a decoupled look-back, 32 bits: a tile's own count, then its
+// inclusive prefix.  Narrow form (fewer than 2^27 keys): the pass number marks
+// the state, so that one array serves all passes without being cleared; wide
+// form: 0 = nothing yet, the array is cleared before each pass.
+struct TileState {
+    uint32_t epoch;
+    int wide;
+    __device__ __forceinline__ uint32_t own(uint32_t c) const
+    {
+        return wide ? c + 1u : (epoch << 28) | c;
     }
-    __syncthreads();
-    hist[(int64_t)tid * tiles + blockIdx.x] = cnt[tid];
+    __device__ __forceinline__ uint32_t incl(uint32_t c) const
+    {
+        return wide ? 0x80000000u | c : (epoch << 28) | 0x08000000u | c;
+    }
+    __device__ __forceinline__ bool empty(uint32_t w) const { return wide ? w == 0u : (w >> 28) != epoch; }
+    __device__ __forceinline__ bool is_incl(uint32_t w) const
+    {
+        return wide ? (w >> 31) != 0u : (w & 0x08000000u) != 0u;
+    }
+    __device__ __forceinline__ uint32_t value(uint32_t w) const
+    {
+        return wide ? ((w >> 31) ? w & 0x7fffffffu : w - 1u) : w & 0x07ffffffu;
+    }
+};
+constexpr int64_t kNarrowKeys = 1ll << 27;
+
+// Polls before a look-back wait gives up (64 ns sleeps: 0.27 s and more).
+constexpr int kSortPolls = 1 << 22;
+
+// Sum of the counts of the tiles before `tile` (stride words apart), by one
+// thread.  False when a wait gave up.
+__device__ __forceinline__ bool tile_prefix(const uint32_t* st, int64_t tile, int stride,
+                                            const TileState& ts, const Header* hdr, uint32_t& prefix)
+{
+    constexpr int kAhead = 8;               // states read at a time: one L2 latency for eight
+    uint32_t sum = 0;
+    for (int64_t t0 = tile - 1; t0 >= 0; t0 -= kAhead) {
+        uint32_t w[kAhead];
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) w[q] = t0 - q >= 0 ? __ldcg(st + (t0 - q) * stride) : 0u;
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q) {
+            const int64_t t = t0 - q;
+            if (t < 0) break;                // (tile 0 publishes an inclusive prefix at once)
+            for (int polls = 0; ts.empty(w[q]); ++polls) {
+                if (polls > kSortPolls || ((polls & 1023) == 1023 && __ldcg(&hdr->err) != kNoError))
+                    return false;
+                if (polls > 8) __nanosleep(64);
+                w[q] = __ldcg(st + t * stride);
+            }
+            sum += ts.value(w[q]);
+            if (ts.is_incl(w[q])) { prefix = sum; return true; }
+        }
+    }
+    prefix = sum;
+    return true;
 }
 
-// Exclusive scan of rows in place: CTA r scans a[r * len .. (r + 1) * len)
-// (256 threads, 256 counters per round with a running carry) and writes the
-// row's total to totals[r] when totals is given.  For the digit histograms a
-// row is one digit's counts over the tiles.
-__global__ void __launch_bounds__(256) scan_rows_kernel(uint32_t* __restrict__ a, int64_t len,
-                                                        uint32_t* __restrict__ totals)
+// Counts of all eight digits; the CTA that finishes last turns them into
+// exclusive scans and plans the passes.  Clears the states of the first pass
+// that needs it and of the rank kernel.
+__global__ void __launch_bounds__(256)
+radix_hist_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ misc,
+                  uint32_t* __restrict__ status, int64_t nstatus, uint32_t* __restrict__ tsum,
+                  int64_t ntsum, const Header* hdr)
 {
+    __shared__ uint32_t cnt[8][256];
     __shared__ uint32_t wsum[8];
-    __shared__ uint32_t carry;
+    __shared__ int last, trivial[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t* row = a + (int64_t)blockIdx.x * len;
-    if (tid == 0) carry = 0;
+    const int64_t gid = (int64_t)blockIdx.x * 256 + tid, gsz = (int64_t)gridDim.x * 256;
+    for (int64_t i = gid; i < nstatus; i += gsz) status[i] = 0;
+    for (int64_t i = gid; i < ntsum; i += gsz) tsum[i] = 0;
+    for (int d = 0; d < 8; ++d) cnt[d][tid] = 0;
     __syncthreads();
-    for (int64_t base = 0; base < len; base += 256) {
-        const int64_t i = base + tid;
-        const uint32_t x = i < len ? row[i] : 0u;
+    const int64_t m = (int64_t)hdr->nkeys;
+    for (int64_t i0 = gid - lane; i0 < m; i0 += gsz) {      // warp-uniform
+        const bool valid = i0 + lane < m;
+        const uint64_t k = key[valid ? i0 + lane : i0];
+        const unsigned live = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const unsigned g = (unsigned)(k >> (8 * d)) & 255u;
+            if (d >= 6) {
+                // sign, exponent and the first mantissa bits: mostly one value per warp
+                const unsigned g0 = __shfl_sync(0xffffffffu, g, 0);
+                if (__all_sync(0xffffffffu, g == g0)) {
+                    if (lane == 0) atomicAdd(&cnt[d][g0], (unsigned)__popc(live));
+                    continue;
+                }
+            }
+            if (valid) atomicAdd(&cnt[d][g], 1u);
+        }
+    }
+    __syncthreads();
+    for (int d = 0; d < 8; ++d)
+        if (cnt[d][tid]) atomicAdd(&misc[d * 256 + tid], cnt[d][tid]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&misc[kMiscDone], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int d = 0; d < 8; ++d) {
+        const uint32_t x = __ldcg(&misc[d * 256 + tid]);
+        const int all = __syncthreads_or((int64_t)x == m);   // one digit holds every key
+        if (tid == 0) trivial[d] = all;
         uint32_t incl = x;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -127,87 +216,137 @@ __global__ void __launch_bounds__(256) scan_rows_kernel(uint32_t* __restrict__ a
         }
         if (lane == 31) wsum[warp] = incl;
         __syncthreads();
-        uint32_t before = carry;
+        uint32_t before = 0;
         for (int w = 0; w < warp; ++w) before += wsum[w];
-        if (i < len) row[i] = before + incl - x;
-        __syncthreads();
-        if (tid == 255) carry = before + incl;
+        misc[d * 256 + tid] = before + incl - x;
         __syncthreads();
     }
-    if (tid == 0 && totals) totals[blockIdx.x] = carry;
-}
-
-// Stable scatter of one tile by the digit at `shift`: the tile's keys are
-// taken in rounds of 256 (key order), ranked within the round by warp match
-// and per-warp digit counts, and written after the positions the digit's
-// earlier keys (earlier tiles, earlier rounds) took.
-__global__ void __launch_bounds__(kSortThreads2)
-radix_scatter_kernel(const uint64_t* __restrict__ kin, const uint32_t* __restrict__ pin,
-                     uint64_t* __restrict__ kout, uint32_t* __restrict__ pout,
-                     const uint32_t* __restrict__ offs, const uint32_t* __restrict__ dbase,
-                     int64_t tiles, int shift, const Header* hdr)
-{
-    __shared__ uint32_t run[256];
-    __shared__ uint16_t wcnt[kSortWarps][256];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t m = (int64_t)hdr->nkeys;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    run[tid] = dbase[tid] + offs[(int64_t)tid * tiles + blockIdx.x];
-    for (int w = 0; w < kSortWarps; ++w) wcnt[w][tid] = 0;
-    __syncthreads();
-    if (base >= m) return;
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = base + (int64_t)r * kSortThreads2 + tid;
-        const bool valid = i < m;
-        uint64_t k = 0;
-        uint32_t p = 0;
-        unsigned d = 256u + lane;            // distinct dummy digits for idle lanes
-        if (valid) {
-            k = kin[i];
-            p = pin[i];
-            d = (unsigned)(k >> shift) & 255u;
-        }
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const unsigned rank = __popc(peers & ((1u << lane) - 1u));
-        if (valid && rank == 0) wcnt[warp][d] = (uint16_t)__popc(peers);
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = run[d] + rank;
-            for (int w = 0; w < warp; ++w) pos += wcnt[w][d];
-            kout[pos] = k;
-            pout[pos] = p;
-        }
-        __syncthreads();
-        {
-            uint32_t tot = 0;
-            for (int w = 0; w < kSortWarps; ++w) { tot += wcnt[w][tid]; wcnt[w][tid] = 0; }
-            run[tid] += tot;
-        }
-        __syncthreads();
-        if (base + (int64_t)(r + 1) * kSortThreads2 >= m) break;   // block-uniform
-    }
-}
-
-// Distinct keys per tile (a key differing from its predecessor, or the first).
-__global__ void __launch_bounds__(kSortThreads2)
-rank_count_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ tsum, const Header* hdr)
-{
-    __shared__ uint32_t wsum[kSortWarps];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t m = (int64_t)hdr->nkeys;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    uint32_t c = 0;
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = base + (int64_t)r * kSortThreads2 + tid;
-        if (i < m) c += (i == 0 || key[i] != key[i - 1]) ? 1u : 0u;
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) wsum[warp] = c;
-    __syncthreads();
     if (tid == 0) {
-        uint32_t s = 0;
-        for (int w = 0; w < kSortWarps; ++w) s += wsum[w];
-        tsum[blockIdx.x] = s;
+        uint32_t src = 0;
+        for (int d = 0; d < 8; ++d) {
+            misc[kMiscPlan + d] = trivial[d] ? 2u : src;
+            if (!trivial[d]) src ^= 1u;
+        }
+        misc[kMiscFinal] = src;
+    }
+}
+
+constexpr size_t radix_pass_smem()
+{
+    return (size_t)kSortTile * 12 + (size_t)kSortWarps * 256 * 2;
+}
+
+// One stable pass by the digit at 8 * pass (see the file's head).
+__global__ void __launch_bounds__(kSortThreads2, 2)
+radix_pass_kernel(uint64_t* __restrict__ key0, uint64_t* __restrict__ key1, uint32_t* __restrict__ pay0,
+                  uint32_t* __restrict__ pay1, uint32_t* __restrict__ status,
+                  uint32_t* __restrict__ misc, int pass, int wide, Header* hdr)
+{
+    extern __shared__ __align__(16) unsigned char rsm[];
+    uint64_t* skey = reinterpret_cast<uint64_t*>(rsm);
+    uint32_t* spay = reinterpret_cast<uint32_t*>(rsm + (size_t)kSortTile * 8);
+    uint16_t* wcnt = reinterpret_cast<uint16_t*>(rsm + (size_t)kSortTile * 12);   // [warp][digit]
+    __shared__ uint32_t dstart[256];      // first place of a digit in the ordered tile
+    __shared__ uint32_t gstart[256];      // its place in the output, minus dstart
+    __shared__ uint32_t wsum[8];
+    __shared__ int64_t s_tile;
+    __shared__ int s_fail;
+    const uint32_t plan = misc[kMiscPlan + pass];
+    if (plan > 1u) return;                                  // all keys share this digit
+    const uint64_t* kin = plan ? key1 : key0;
+    const uint32_t* pin = plan ? pay1 : pay0;
+    uint64_t* kout = plan ? key0 : key1;
+    uint32_t* pout = plan ? pay0 : pay1;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const TileState ts{(uint32_t)pass + 1u, wide};
+    if (tid == 0) {
+        s_tile = (int64_t)atomicAdd(&misc[kMiscTicket + pass], 1u);
+        s_fail = 0;
+    }
+    for (int i = tid; i < kSortWarps * 256 / 2; i += kSortThreads2) reinterpret_cast<uint32_t*>(wcnt)[i] = 0;
+    __syncthreads();
+    const int64_t tile = s_tile, m = (int64_t)hdr->nkeys;
+    const int64_t base = tile * kSortTile;
+    if (base >= m) return;                                  // nor any tile after it
+    const int cnt = m - base < kSortTile ? (int)(m - base) : kSortTile;
+    const int shift = 8 * pass;
+    // warp w holds the tile's keys w * 512 .., item j of lane l is key 32 j + l
+    // of them; past the end: all ones, which order after every key of the tile
+    const int wbase = warp * 32 * kSortItems + lane;
+    uint64_t k[kSortItems];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const int i = wbase + 32 * j;
+        k[j] = i < cnt ? kin[base + i] : ~0ull;
+    }
+    uint16_t* my = wcnt + warp * 256;
+    uint32_t rank2[kSortItems / 2];                         // 16-bit ranks in the warp's digit
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const unsigned d = (unsigned)(k[j] >> shift) & 255u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const unsigned before = my[d];
+        const unsigned r = before + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if ((__ffs(peers) - 1) == lane) my[d] = (uint16_t)(before + __popc(peers));
+        __syncwarp();
+        if (j & 1) rank2[j / 2] |= r << 16; else rank2[j / 2] = r;
+    }
+    __syncthreads();
+    // per digit: places of the warps, the tile's count, its prefix
+    uint32_t total = 0;
+    if (tid < 256) {
+        for (int w = 0; w < kSortWarps; ++w) {
+            const uint32_t c = wcnt[w * 256 + tid];
+            wcnt[w * 256 + tid] = (uint16_t)total;
+            total += c;
+        }
+        const uint32_t real = total - (tid == 255 ? (uint32_t)(kSortTile - cnt) : 0u);
+        uint32_t* st = status + tid;
+        atomicExch(st + tile * 256, tile == 0 ? ts.incl(real) : ts.own(real));
+        uint32_t incl = total;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        dstart[tid] = incl - total;                         // within the warp, for now
+        uint32_t prefix = 0;
+        if (tile > 0) {
+            if (tile_prefix(st, tile, 256, ts, hdr, prefix))
+                atomicExch(st + tile * 256, ts.incl(prefix + real));
+            else
+                s_fail = 1;
+        }
+        gstart[tid] = misc[pass * 256 + tid] + prefix;
+    }
+    __syncthreads();
+    if (tid < 256) {
+        uint32_t before = 0;
+        for (int w = 0; w < warp; ++w) before += wsum[w];
+        dstart[tid] += before;
+        gstart[tid] -= dstart[tid];
+    }
+    if (s_fail) {                                           // block-uniform
+        if (tid == 0) record_error(hdr, kErrWait, tile);
+        return;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const unsigned d = (unsigned)(k[j] >> shift) & 255u;
+        const uint32_t r = (j & 1) ? rank2[j / 2] >> 16 : rank2[j / 2] & 0xffffu;
+        const uint32_t pos = dstart[d] + my[d] + r;         // < kSortTile
+        skey[pos] = k[j];
+        const int i = wbase + 32 * j;
+        if (i < cnt) spay[pos] = pin[base + i];
+    }
+    __syncthreads();
+    for (int i = tid; i < cnt; i += kSortThreads2) {
+        const uint64_t kk = skey[i];
+        const uint32_t at = gstart[(unsigned)(kk >> shift) & 255u] + (uint32_t)i;
+        kout[at] = kk;
+        pout[at] = spay[i];
     }
 }
 
@@ -215,53 +354,82 @@ rank_count_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ tsum,
 // written into the rank field of the packed element its payload names
 // (bit 31 selects the set: 0 = set0, 1 = set1).
 __global__ void __launch_bounds__(kSortThreads2)
-rank_write_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ pay,
-                  const uint32_t* __restrict__ tsum, KElem* pack0, KElem* pack1, const Header* hdr)
+rank_write_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict__ key1,
+                  const uint32_t* __restrict__ pay0, const uint32_t* __restrict__ pay1,
+                  uint32_t* __restrict__ tsum, uint32_t* __restrict__ misc, KElem* pack0, KElem* pack1,
+                  Header* hdr)
 {
-    __shared__ uint32_t wsum[kSortWarps];
-    __shared__ uint32_t carry;
+    __shared__ uint32_t wcount[kSortWarps];
+    __shared__ uint32_t s_prefix;
+    __shared__ int64_t s_tile;
+    __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t m = (int64_t)hdr->nkeys;
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    if (tid == 0) carry = tsum[blockIdx.x];
+    const bool one = misc[kMiscFinal] != 0u;
+    const uint64_t* key = one ? key1 : key0;
+    const uint32_t* pay = one ? pay1 : pay0;
+    if (tid == 0) {
+        s_tile = (int64_t)atomicAdd(&misc[kMiscTicket + 8], 1u);
+        s_fail = 0;
+    }
     __syncthreads();
-    for (int r = 0; r < kSortItems; ++r) {
-        if (base + (int64_t)r * kSortThreads2 >= m) break;          // block-uniform
-        const int64_t i = base + (int64_t)r * kSortThreads2 + tid;
-        const uint32_t f = (i < m && (i == 0 || key[i] != key[i - 1])) ? 1u : 0u;
-        uint32_t incl = f;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+    const int64_t tile = s_tile, m = (int64_t)hdr->nkeys;
+    const int64_t base = tile * kSortTile;
+    if (base >= m) return;
+    const int64_t w0 = base + warp * 32 * kSortItems;       // the warp's keys, in order
+    uint32_t heads[kSortItems];                             // ballots: key differs from the one before
+    uint32_t count = 0;
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const int64_t i = w0 + 32 * j + lane;
+        const uint64_t k = i < m ? key[i] : 0;
+        uint64_t kp = __shfl_up_sync(0xffffffffu, k, 1);
+        if (lane == 0 && i > 0 && i < m) kp = key[i - 1];
+        heads[j] = __ballot_sync(0xffffffffu, i < m && (i == 0 || k != kp));
+        count += __popc(heads[j]);
+    }
+    if (lane == 0) wcount[warp] = count;
+    __syncthreads();
+    if (tid == 0) {
+        const TileState ts{0u, 1};
+        uint32_t total = 0, prefix = 0;
+        for (int w = 0; w < kSortWarps; ++w) { const uint32_t c = wcount[w]; wcount[w] = total; total += c; }
+        atomicExch(tsum + tile, tile == 0 ? ts.incl(total) : ts.own(total));
+        if (tile > 0) {
+            if (tile_prefix(tsum, tile, 1, ts, hdr, prefix)) atomicExch(tsum + tile, ts.incl(prefix + total));
+            else s_fail = 1;
         }
-        if (lane == 31) wsum[warp] = incl;
-        __syncthreads();
-        uint32_t before = carry;
-        for (int w = 0; w < warp; ++w) before += wsum[w];
+        s_prefix = prefix;
+    }
+    __syncthreads();
+    if (s_fail) {                                           // block-uniform
+        if (tid == 0) record_error(hdr, kErrWait, tile);
+        return;
+    }
+    uint32_t before = s_prefix + wcount[warp];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const int64_t i = w0 + 32 * j + lane;
         if (i < m) {
-            const uint32_t d = before + incl;     // distinct keys in [0, i]
+            const uint32_t d = before + __popc(heads[j] & (0xffffffffu >> (31 - lane)));
             const uint32_t p = pay[i];
             KElem* dst = (p >> 31) ? pack1 : pack0;
             dst[p & 0x7fffffffu].k = 2u * d;
         }
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t s = 0;
-            for (int w = 0; w < kSortWarps; ++w) s += wsum[w];
-            carry += s;
-        }
-        __syncthreads();
+        before += __popc(heads[j]);
     }
 }
 
 // Keys of the integration bounds a and b (one thread): 2 * (distinct ends
 // below q) + 1, or + 2 when q is itself an interval end; b = inf maps to the
 // rank of the last intervals.  Written to hdr->bound_key[0..1].
-__global__ void bound_keys_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ pay,
-                                  const KElem* pack0, const KElem* pack1, double a, double b,
+__global__ void bound_keys_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict__ key1,
+                                  const uint32_t* __restrict__ pay0, const uint32_t* __restrict__ pay1,
+                                  const uint32_t* __restrict__ misc, const KElem* pack0, const KElem* pack1, double a, double b,
                                   Header* hdr)
 {
     const int64_t m = (int64_t)hdr->nkeys;
+    const uint64_t* key = misc[kMiscFinal] ? key1 : key0;
+    const uint32_t* pay = misc[kMiscFinal] ? pay1 : pay0;
     const double q2[2] = {a, b};
     for (int w = 0; w < 2; ++w) {
         const double q = q2[w];
@@ -284,32 +452,36 @@ __global__ void bound_keys_kernel(const uint64_t* __restrict__ key, const uint32
 cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int64_t n0,
                       KElem* pack1, const int64_t* poff1, int64_t n1, Header* hdr, cudaStream_t s)
 {
-    count_keys_kernel<<<1, 1, 0, s>>>(hdr, poff0, n0, poff1, n1);
-    const int64_t tiles = ks.tiles;
-    int src = 0;
+    count_keys_kernel<<<1, 256, 0, s>>>(hdr, poff0, n0, poff1, n1, ks.misc);
+    const unsigned tiles = (unsigned)ks.tiles;
+    const int wide = ks.cap >= kNarrowKeys ? 1 : 0;
+    cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)radix_pass_smem());
+    if (e != cudaSuccess) return e;
+    // a CTA per 2,048 keys up to four per SM
+    int64_t hgrid = (ks.cap + 2047) / 2048;
+    const int64_t hcap = (int64_t)device_sm_count() * 4;
+    if (hgrid > hcap) hgrid = hcap;
+    if (hgrid < 1) hgrid = 1;
+    radix_hist_kernel<<<(unsigned)hgrid, 256, 0, s>>>(ks.key[0], ks.misc, ks.status, ks.tiles * 256,
+                                                      ks.tsum, ks.tiles + 1, hdr);
     for (int pass = 0; pass < 8; ++pass) {
-        const int shift = 8 * pass;
-        radix_hist_kernel<<<(unsigned)tiles, kSortThreads2, 0, s>>>(ks.key[src], ks.hist, tiles, shift, hdr);
-        // each digit's counts over the tiles, then the digit totals
-        scan_rows_kernel<<<256, 256, 0, s>>>(ks.hist, tiles, ks.dsum);
-        scan_rows_kernel<<<1, 256, 0, s>>>(ks.dsum, 256, nullptr);
-        radix_scatter_kernel<<<(unsigned)tiles, kSortThreads2, 0, s>>>(
-            ks.key[src], ks.pay[src], ks.key[1 - src], ks.pay[1 - src], ks.hist, ks.dsum, tiles,
-            shift, hdr);
-        src = 1 - src;
+        if (wide && pass > 0) {
+            e = cudaMemsetAsync(ks.status, 0, sizeof(uint32_t) * 256 * (size_t)ks.tiles, s);
+            if (e != cudaSuccess) return e;
+        }
+        radix_pass_kernel<<<tiles, kSortThreads2, radix_pass_smem(), s>>>(
+            ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.status, ks.misc, pass, wide, hdr);
     }
-    rank_count_kernel<<<(unsigned)tiles, kSortThreads2, 0, s>>>(ks.key[src], ks.tsum, hdr);
-    scan_rows_kernel<<<1, 256, 0, s>>>(ks.tsum, tiles, nullptr);
-    rank_write_kernel<<<(unsigned)tiles, kSortThreads2, 0, s>>>(ks.key[src], ks.pay[src], ks.tsum,
-                                                                pack0, pack1, hdr);
-    static_assert((8 & 1) == 0, "an even number of passes leaves the sorted keys in key[0]");
+    rank_write_kernel<<<tiles, kSortThreads2, 0, s>>>(ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.tsum,
+                                                      ks.misc, pack0, pack1, hdr);
     return cudaGetLastError();
 }
 
 cudaError_t bound_keys(const KeySort& ks, const KElem* pack0, const KElem* pack1, double a, double b,
                        Header* hdr, cudaStream_t s)
 {
-    bound_keys_kernel<<<1, 1, 0, s>>>(ks.key[0], ks.pay[0], pack0, pack1, a, b, hdr);
+    bound_keys_kernel<<<1, 1, 0, s>>>(ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.misc, pack0, pack1, a, b, hdr);
     return cudaGetLastError();
 }
 

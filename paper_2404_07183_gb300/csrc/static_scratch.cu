@@ -27,7 +27,9 @@
 
 namespace {
 
-__device__ __align__(256) unsigned char g_noalloc_scratch[PCF_NOALLOC_SCRATCH_BYTES];
+// kKeySortExtra on top: sort counters that the limit on inputs does not count.
+constexpr size_t kScratchBytes = (size_t)PCF_NOALLOC_SCRATCH_BYTES + pcfgb::kKeySortExtra;
+__device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 void* g_scratch_ptr[kMaxDevices] = {};
@@ -58,10 +60,13 @@ extern "C" int pcf_pairwise_noalloc(const pcf_csr* x, const pcf_integral* F, int
     size_t need = 0;
     int rc = pcf_workspace_size(x, nullptr, precision, PCF_WS_FORWARD, &need);
     if (rc != PCF_OK) return rc;
-    if (need > (size_t)PCF_NOALLOC_SCRATCH_BYTES) return PCF_ENOWS;
+    size_t limit = (size_t)PCF_NOALLOC_SCRATCH_BYTES;
+    if (x->dtype == PCF_F64 && (precision & 0xff) != PCF_PREC_F64 && !(precision & PCF_PREC_ROUND_TIMES))
+        limit = kScratchBytes;                       // the keyed form's sort
+    if (need > limit) return PCF_ENOWS;
     void* scratch = nullptr;
     rc = scratch_address(&scratch);
     if (rc != PCF_OK) return rc;
     return pcf_pairwise(x, F, nF, precision, layout, out_dtype, 0, scratch,
-                        (size_t)PCF_NOALLOC_SCRATCH_BYTES, stream);
+                        kScratchBytes, stream);
 }
