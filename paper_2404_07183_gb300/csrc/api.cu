@@ -42,6 +42,7 @@ __global__ void init_header_kernel(Header* h, int keep_set1)
     h->maxlen[0] = 0;
     if (!keep_set1) h->maxlen[1] = 0;
     h->need64 = keep_set1 ? (h->need64 & 2u) : 0u;   // a reused set 1 keeps its need
+    h->wild = keep_set1 ? (h->wild & 2u) : 0u;
     h->tiles = 0;
 }
 

@@ -59,7 +59,8 @@ struct Header {
     unsigned int bound_key[2];   // keyed walks: order keys of the bounds a, b
     unsigned int need64;         // PCF_PREC_AUTO64: bit s set when set s needs the
                                  // float64 walk (range or time resolution)
-    unsigned int pad32;
+    unsigned int wild;           // bit s: a value of set s lies outside the range of the
+                                 // integer products of float64 walks (f64int.cuh)
     unsigned long long pad[26];
 };
 static_assert(sizeof(Header) == 256, "header is 256 bytes");

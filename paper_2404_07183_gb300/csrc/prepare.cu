@@ -9,6 +9,7 @@
 #include <cfloat>
 #include <cmath>
 
+#include "f64int.cuh"
 #include "internal.cuh"
 
 namespace pcfgb {
@@ -22,7 +23,8 @@ __device__ __forceinline__ bool finite_val(T x) { return isfinite(x); }
 // auto64 (float64 input, PCF_PREC_AUTO64): instead of rejecting a time or
 // value outside float32's range, mark the set as needing the float64 walk
 // (Header::need64 bit `slot`), likewise for nonzero values below FLT_MIN and
-// for gaps below 2^-30 of their time.
+// for gaps below 2^-30 of their time.  Values outside the range of the float64
+// walks' integer products are noted in Header::wild.
 template <typename T>
 __global__ void validate_kernel(const int64_t* __restrict__ offsets,
                                 const T* __restrict__ times, const T* __restrict__ values,
@@ -33,7 +35,7 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
     // a collection built by an earlier kernel of the call is only checked
     // when that kernel ran (no error recorded before it)
     if (skip_on_error && hdr->err != kNoError) return;
-    bool need64 = false;
+    bool need64 = false, wild = false;
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -66,6 +68,8 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
             const T t = times[k];
             const T v = values[k];
             const T tp = k > o0 ? times[k - 1] : T(0);
+            // (every finite float32 suits)
+            if constexpr (sizeof(T) == 8) wild |= !f64i_value_suits((uint64_t)__double_as_longlong(v));
             if (!finite_val(t)) { record_error(hdr, kErrTimeNaN, k); continue; }
             if (!finite_val(v)) { record_error(hdr, kErrValueNaN, k); continue; }
             if (k == o0) {
@@ -89,6 +93,7 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
         }
     }
     if (__any_sync(0xffffffffu, need64) && lane == 0) atomicOr(&hdr->need64, 1u << slot);
+    if (__any_sync(0xffffffffu, wild) && lane == 0) atomicOr(&hdr->wild, 1u << slot);
     // warp max then one atomic per warp
     for (int o = 16; o > 0; o >>= 1) local_max = max(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
     if (lane == 0 && local_max) atomicMax(&hdr->maxlen[slot], local_max);

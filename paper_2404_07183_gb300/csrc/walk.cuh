@@ -49,6 +49,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "f64int.cuh"
 #include "internal.cuh"
 
 namespace pcfgb {
@@ -90,15 +91,34 @@ template <> struct WalkForm<float, true> {
     static __device__ __forceinline__ float val(const E& e) { return e.v; }
 };
 
+// Products and interval widths of a walk; INT: float64 ones on the integer
+// pipes (the same bits, for the operands f64int.cuh states).
+template <bool INT, typename T>
+__device__ __forceinline__ T walk_mul(T a, T b)
+{
+    if constexpr (INT)
+        return __longlong_as_double((long long)f64i_mul((uint64_t)__double_as_longlong(a),
+                                                        (uint64_t)__double_as_longlong(b)));
+    else return a * b;
+}
+template <bool INT, typename T>
+__device__ __forceinline__ T walk_width(T n, T c)
+{
+    if constexpr (INT)
+        return __longlong_as_double((long long)f64i_width((uint64_t)__double_as_longlong(n),
+                                                          (uint64_t)__double_as_longlong(c)));
+    else return n - c;
+}
+
 // h(a, b) of Sec. 2.2 for one metric, in the walk type.
-template <int MI, typename T>
+template <int MI, bool INT, typename T>
 __device__ __forceinline__ T term_h(T a, T b, T d, T p)
 {
     if constexpr (MI == MI_L1) return fabs(d);
-    else if constexpr (MI == MI_L2) return d * d;
-    else if constexpr (MI == MI_L3) { T ad = fabs(d); return ad * ad * ad; }
+    else if constexpr (MI == MI_L2) return walk_mul<INT>(d, d);
+    else if constexpr (MI == MI_L3) { T ad = fabs(d); return walk_mul<INT>(ad, ad) * ad; }
     else if constexpr (MI == MI_LP) return pow(fabs(d), p);
-    else return a * b;
+    else return walk_mul<INT>(a, b);
 }
 
 template <int PREC> struct Acc;
@@ -167,13 +187,13 @@ template <> struct Acc<kF32B> {
     }
 };
 
-template <int COMBO, int PREC, typename T>
+template <int COMBO, int PREC, typename T, bool INT = false>
 __device__ __forceinline__ void accumulate(Acc<PREC>* acc, T a, T b, T dt, T p)
 {
     const T d = a - b;
-    acc[0].add(term_h<combo_metric(COMBO, 0)>(a, b, d, p), dt);
-    if constexpr (combo_n(COMBO) > 1) acc[1].add(term_h<combo_metric(COMBO, 1)>(a, b, d, p), dt);
-    if constexpr (combo_n(COMBO) > 2) acc[2].add(term_h<combo_metric(COMBO, 2)>(a, b, d, p), dt);
+    acc[0].add(term_h<combo_metric(COMBO, 0), INT>(a, b, d, p), dt);
+    if constexpr (combo_n(COMBO) > 1) acc[1].add(term_h<combo_metric(COMBO, 1), INT>(a, b, d, p), dt);
+    if constexpr (combo_n(COMBO) > 2) acc[2].add(term_h<combo_metric(COMBO, 2), INT>(a, b, d, p), dt);
 }
 
 // Accumulators of one walk.  The generic form keeps one Acc per metric.
@@ -181,8 +201,11 @@ template <int PREC, int COMBO>
 struct AccSet {
     static constexpr int NM = combo_n(COMBO);
     Acc<PREC> a[NM];
-    template <typename T>
-    __device__ __forceinline__ void add(T va, T vb, T dt, T p) { accumulate<COMBO, PREC>(a, va, vb, dt, p); }
+    template <bool INT = false, typename T>
+    __device__ __forceinline__ void add(T va, T vb, T dt, T p)
+    {
+        accumulate<COMBO, PREC, T, INT>(a, va, vb, dt, p);
+    }
     __device__ __forceinline__ void flush()
     {
 #pragma unroll
@@ -196,9 +219,9 @@ struct AccSet {
     {
         Terms t;
         const T d = va - vb;
-        t.h[0] = term_h<combo_metric(COMBO, 0)>(va, vb, d, p);
-        if constexpr (NM > 1) t.h[1] = term_h<combo_metric(COMBO, 1)>(va, vb, d, p);
-        if constexpr (NM > 2) t.h[2] = term_h<combo_metric(COMBO, 2)>(va, vb, d, p);
+        t.h[0] = term_h<combo_metric(COMBO, 0), false>(va, vb, d, p);
+        if constexpr (NM > 1) t.h[1] = term_h<combo_metric(COMBO, 1), false>(va, vb, d, p);
+        if constexpr (NM > 2) t.h[2] = term_h<combo_metric(COMBO, 2), false>(va, vb, d, p);
         return t;
     }
     __device__ __forceinline__ void add_terms(const Terms& t, float dt)
@@ -429,6 +452,16 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     static_assert(THREADS == 1024 || THREADS == 512, "thread count");
     static_assert(!KEYED || sizeof(T) == 4, "keyed walks are float32 walks");
 
+    // float64 walks form widths and products on the integer pipes, which run
+    // beside the float64 pipe that bounds them (L1 three operations per step,
+    // two of them left there; L1 + L2 + Gram seven, four left).  Walk alone,
+    // 2,501 stable-rank curves: L1 11.2 -> 7.5 ms, L2 15.0 -> 7.9, Gram 11.2 ->
+    // 7.7, the three fused 25.3 -> 14.4; 1,000 curves of 55 points, L1 0.41 ->
+    // 0.29 ms.  A fallback inside the step does not do: a float64 instruction
+    // holds its pipe with all lanes predicated off too.  (Not in the weighted
+    // walks, whose exponentials dominate, nor in the 40-register schedules.)
+    constexpr bool kInt = sizeof(T) == 8 && WEIGHT == 0 && CTAS < 3;
+
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int32_t sS[kTilePcfs], sNext[kTilePcfs], sLen[kTilePcfs], sStaged[kTilePcfs];
     __shared__ int64_t sOff[kTilePcfs];
@@ -461,6 +494,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     auto split_wc = [W](int c, int wr) { return (NR * W - 2 * wr) / RC; };
     auto split_ok = [](int wr, int wc) { return wr >= 4 && wc >= 4; };
     const T p0 = (T)a.p[0];
+    // a value of the call's collections does not suit the integer products
+    const bool wild = kInt && a.hdr->wild != 0u;
     const unsigned smem_base = (unsigned)__cvta_generic_to_shared(smem);
     const E* packR = reinterpret_cast<const E*>(a.pack_r);
     const E* packC = reinterpret_cast<const E*>(a.pack_c);
@@ -761,22 +796,45 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
                     }
                 } else {
                     T tf = ef.x, tg = eg.x, vf = ef.y, vg = eg.y;
-#define PCF_WALK_STEP()                                                           \
+#define PCF_WALK_STEP(INT)                                                        \
                     {                                                             \
                         const T tn = first_end(tf, tg);                           \
-                        const T dt = weight_span<WEIGHT>(tc, tn - tc, lam, inv_lam); \
+                        const T dt = weight_span<WEIGHT>(tc, walk_width<INT>(tn, tc), lam, inv_lam); \
                         tc = tn;                                                  \
-                        acc.add(vf, vg, dt, p0);                                  \
+                        acc.template add<INT>(vf, vg, dt, p0);                    \
                         advance_cursor<kRow>(af, tf, vf, ag, tg, vg);             \
+                    }
+                    if constexpr (kInt) {
+                        // the pair's last end before T1 bounds the ends to come: from
+                        // 2^-10 of it on the widths suit the integer form, until then
+                        // (one or two steps as a rule) the float64 pipe forms them
+                        const int lf = sNext[pf] - sS[pf], lg = sNext[pg] - sS[pg];
+                        long long tm = 0;
+                        if (lf > 0) tm = __double_as_longlong(reinterpret_cast<const E*>(
+                            smem + base_f + (unsigned)(lf - 1) * kRow)->x);
+                        if (lg > 0) {
+                            const long long t = __double_as_longlong(reinterpret_cast<const E*>(
+                                smem + base_g + (unsigned)(lg - 1) * kRow)->x);
+                            tm = t > tm ? t : tm;
+                        }
+                        const uint32_t em = (uint32_t)(tm >> 52);
+                        const bool suits = !wild && em >= kWidthExpLo && em <= kWidthExpHi;
+                        const long long from = suits ? tm - ((long long)kWidthOctaves << 52)
+                                                     : 0x7fffffffffffffffll;
+#pragma unroll 1
+                        while (cnt > 0 && __double_as_longlong(tc) < from) {
+                            PCF_WALK_STEP(false)
+                            --cnt;
+                        }
                     }
 #pragma unroll 1
                     for (; cnt >= kUnroll; cnt -= kUnroll) {
 #pragma unroll
-                        for (int u = 0; u < kUnroll; ++u) PCF_WALK_STEP()
+                        for (int u = 0; u < kUnroll; ++u) PCF_WALK_STEP(kInt)
                         acc.flush();
                     }
 #pragma unroll 1
-                    for (; cnt > 0; --cnt) PCF_WALK_STEP()
+                    for (; cnt > 0; --cnt) PCF_WALK_STEP(kInt)
 #undef PCF_WALK_STEP
                     if (last && bounded) {
                         // closing rectangle [tc, hi) with the values holding at hi
