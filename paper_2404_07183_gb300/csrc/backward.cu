@@ -17,7 +17,9 @@
 // summed with float64 atomics into packed-order accumulators, then scattered
 // back to the input order.
 #include <cmath>
+#include <type_traits>
 
+#include "f64int.cuh"
 #include "internal.cuh"
 
 namespace pcfgb {
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(1024) backward_kernel(const BackArgs a)
     if (a.hdr->err != kNoError) return;
     const int r = threadIdx.x >> 5, c = threadIdx.x & 31;
     const int64_t NB = a.nb;
+    const bool wild = a.hdr->wild != 0u;
     for (int64_t u = blockIdx.x;; u += gridDim.x) {
         const int64_t t = a.shard_index + u * a.shard_count;   // this shard's tiles
         if (t >= a.ntiles) break;
@@ -114,38 +117,58 @@ __global__ void __launch_bounds__(1024) backward_kernel(const BackArgs a)
         // Alg. 1 walk over [0, inf) with simultaneous advance on ties.  End
         // times are compared by their bit patterns on the integer pipe
         // (non-negative doubles order like their bits; +inf marks the tail).
-        // For L1, L2 and the Gram the value gradients of both sides share one
-        // product, and the time gradient h(v_old, g) - h(v_new, g) is taken
-        // in factored form; every integrand is symmetric, h(a, b) = h(b, a),
-        // so the side that advances (f on a tie) is handled by one
-        // branch-free update with selected operands and addresses -- lanes
-        // of a warp advancing different sides no longer run two half-empty
-        // branches -- and the second side of a shared breakpoint by a rare
-        // extra branch.  float64 operations per rectangle: L2 9, Gram 7, L1 7.
+        // Every integrand is symmetric, h(a, b) = h(b, a), so the side that
+        // advances (f on a tie) is handled by one branch-free update with
+        // selected operands and addresses -- lanes of a warp advancing
+        // different sides do not run two half-empty branches -- and the
+        // second side of a shared breakpoint by a rare extra branch.
+        //
+        // The float64 pipe bounds this walk, so it gets as few operations as
+        // the float64 results allow.  For L1 and L2 the new difference of the
+        // advancing side, bb = v_new - other, is the next rectangle's d (up to
+        // sign), the value gradients collect d * dt (L2) and are scaled once
+        // when they are handed over, and the widths and the square of bb are
+        // formed on the integer pipes (f64int.cuh; the same bits), from the
+        // first end on that is at least 2^-10 of the pair's last one.  That
+        // leaves six operations per rectangle on the float64 pipe (L2 nine,
+        // Gram and L1 seven before).  The adjoint of L2 over 2,048 curves of
+        // 20 to 200 points: 8.5 -> 6.9 ms.
         int kf = 0, kg = 0;
         double2 ef = a.pack[of], eg = a.pack[og];
         double tc = 0.0, gvf = 0.0, gvg = 0.0;
         const long long kInfBits = 0x7ff0000000000000ll;
         const double w2 = 2.0 * w;
-        for (;;) {
+        double d = ef.y - eg.y;                     // L1, L2: v_f - v_g
+        const double gscale = METRIC == PCF_L2 ? w2 : 1.0;
+        long long from = 0x7fffffffffffffffll;      // the integer forms start here
+        if (!wild) {
+            const int ng = a.slen[gj];
+            long long tm = nf > 1 ? __double_as_longlong(a.pack[of + nf - 2].x) : 0;
+            const long long tg = ng > 1 ? __double_as_longlong(a.pack[og + ng - 2].x) : 0;
+            tm = tg > tm ? tg : tm;
+            const uint32_t em = (uint32_t)(tm >> 52);
+            if (em >= kWidthExpLo && em <= kWidthExpHi) from = tm - ((long long)kWidthOctaves << 52);
+        }
+        // one rectangle and advance; false at the tails
+        auto step = [&](auto int_c) -> bool {
+            constexpr bool INT = decltype(int_c)::value;
             const long long bf = __double_as_longlong(ef.x), bg = __double_as_longlong(eg.x);
             const bool sf = bf <= bg;               // f advances (also on a tie)
             const long long bn = sf ? bf : bg;
-            if (bn == kInfBits) break;
+            if (bn == kInfBits) return false;
             const bool tie = bf == bg;
             const double tn = __longlong_as_double(bn);
-            const double dt = tn - tc;
+            const double dt = INT ? __longlong_as_double((long long)f64i_width(
+                                        (uint64_t)bn, (uint64_t)__double_as_longlong(tc)))
+                                  : tn - tc;
             const double vf = ef.y, vg = eg.y;
             const int64_t at = sf ? of + kf : og + kg;   // advancing side's current element
             const double2 nx = a.pack[at + 1];
             const double v_old = sf ? vf : vg, other = sf ? vg : vf;
-            double d = 0.0;
             if constexpr (METRIC == PCF_L2) {
-                // dh/dv_f = 2 d = -dh/dv_g
-                d = vf - vg;
-                const double e = d * dt;
-                gvf = fma(w2, e, gvf);
-                gvg = fma(-w2, e, gvg);
+                // dh/dv_f = 2 d = -dh/dv_g (times w when handed over)
+                gvf = fma(d, dt, gvf);
+                gvg = fma(-d, dt, gvg);
             } else if constexpr (METRIC == PCF_GRAM) {
                 // dh/dv_f = v_g, dh/dv_g = v_f
                 const double wdt = w * dt;
@@ -153,7 +176,6 @@ __global__ void __launch_bounds__(1024) backward_kernel(const BackArgs a)
                 gvg = fma(wdt, vf, gvg);
             } else if constexpr (METRIC == PCF_L1) {
                 // dh/dv_f = sign(d) = -dh/dv_g, 0 where d = 0
-                d = vf - vg;
                 const long long db = __double_as_longlong(d);
                 const double wdt = w * dt;
                 const double sw = (db << 1) == 0 ? 0.0 : (db < 0 ? -wdt : wdt);
@@ -163,27 +185,45 @@ __global__ void __launch_bounds__(1024) backward_kernel(const BackArgs a)
                 gvf += w * bw_dh<METRIC>(vf, vg, a.p) * dt;
                 gvg += w * bw_dh<METRIC>(vg, vf, a.p) * dt;
             }
-            // h(v_old, other) - h(v_new, other) for the advancing side
-            auto tgrad = [&](double vo, double vn, double ot) -> double {
-                if constexpr (METRIC == PCF_L2) { const double bb = vn - ot; return fma(d, d, -(bb * bb)); }
-                else if constexpr (METRIC == PCF_GRAM) return (vo - vn) * ot;
-                else if constexpr (METRIC == PCF_L1) return fabs(d) - fabs(vn - ot);
+            // h(v_old, other) - h(v_new, other) for the advancing side; bb = v_new - other
+            auto tgrad = [&](double vo, double vn, double ot, double bb) -> double {
+                if constexpr (METRIC == PCF_L2) {
+                    const double q = INT ? __longlong_as_double((long long)f64i_mul(
+                                               (uint64_t)__double_as_longlong(bb),
+                                               (uint64_t)__double_as_longlong(bb)))
+                                         : bb * bb;
+                    return fma(d, d, -q);
+                } else if constexpr (METRIC == PCF_GRAM) return (vo - vn) * ot;
+                else if constexpr (METRIC == PCF_L1) return fabs(d) - fabs(bb);
                 else return bw_h<METRIC>(vo, ot, a.p) - bw_h<METRIC>(vn, ot, a.p);
             };
-            atomicAdd(&a.gv[at], sf ? gvf : gvg);
-            atomicAdd(&a.gt[at + 1], w * tgrad(v_old, nx.y, other));
+            constexpr bool kDiff = METRIC == PCF_L1 || METRIC == PCF_L2;
+            const double bb = kDiff ? nx.y - other : 0.0;
+            const double gvs = sf ? gvf : gvg;
+            atomicAdd(&a.gv[at], METRIC == PCF_L2 ? gscale * gvs : gvs);
+            atomicAdd(&a.gt[at + 1], w * tgrad(v_old, nx.y, other, bb));
+            double dn = sf ? bb : -bb;
             if (sf) { gvf = 0.0; ++kf; ef = nx; } else { gvg = 0.0; ++kg; eg = nx; }
             if (tie) {
                 // shared breakpoint: g advances too, against f's value before it
                 const double2 ng = a.pack[og + kg + 1];
-                atomicAdd(&a.gv[og + kg], gvg);
-                atomicAdd(&a.gt[og + kg + 1], w * tgrad(vg, ng.y, vf));
+                const double bg2 = kDiff ? ng.y - vf : 0.0;
+                atomicAdd(&a.gv[og + kg], METRIC == PCF_L2 ? gscale * gvg : gvg);
+                atomicAdd(&a.gt[og + kg + 1], w * tgrad(vg, ng.y, vf, bg2));
                 gvg = 0.0;
                 ++kg;
                 eg = ng;
+                dn = ef.y - eg.y;
             }
+            d = dn;
             tc = tn;
-        }
+            return true;
+        };
+        bool more = true;
+        while (more && __double_as_longlong(tc) < from) more = step(std::false_type{});
+        while (more) more = step(std::true_type{});
+        gvf *= gscale;
+        gvg *= gscale;
         // tail [t_last, inf): infinite width, finite only where dh = 0
         const double df = bw_dh<METRIC>(ef.y, eg.y, a.p), dg = bw_dh<METRIC>(eg.y, ef.y, a.p);
         if (df != 0.0) gvf += w * df * INFINITY;
