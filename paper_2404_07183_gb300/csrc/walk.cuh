@@ -475,7 +475,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     __shared__ K sT1part[2][kSplits];
     __shared__ int sSplit;                          // split of the staged windows
     __shared__ int64_t sUnit;
-    __shared__ int64_t sBlock[CTAS < 3 ? 2 : 1];    // the unit's row and column block
+    __shared__ int64_t sBlock[2];                   // the unit's row and column block
 
     if (gated_off(a.gate, a.gate_want64)) return;   // the other walk of an AUTO64 call
     if (block_sees_error(a.hdr)) return;
@@ -537,10 +537,12 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
 
     // Work units.  Thread 0 takes the next ticket while this unit is walked
     // and decodes a unit for the CTA (decoded by every thread, a unit cost the
-    // CTA about 400 warp instructions and an atomic's latency).  The three-CTA
-    // schedules have no register for the ticket in flight: every thread
-    // decodes there.
-    constexpr bool kLean = CTAS < 3;
+    // CTA about 400 warp instructions and an atomic's latency; the Gram of
+    // 30,000 log-normal curves 82.0 -> 75.9 ms on two CTAs per SM).  Of the
+    // 40-register schedules only the L1, L2 and Gram walks of 8-byte elements
+    // have room for it (74.2 -> 71.5 ms); in the others every thread decodes.
+    constexpr bool kLean = CTAS < 3 || (sizeof(E) == 8 && (COMBO == kComboL1 || COMBO == kComboL2 ||
+                                                         COMBO == kComboGram));
     unsigned long long ticket = 0;
     if (kLean && tid == 0) ticket = atomicAdd(&a.hdr->tiles, 1ull);
     for (;;) {
