@@ -38,6 +38,7 @@ size_t walk_smem_bytes(int window, int elem_bytes)
 
 __global__ void init_header_kernel(Header* h, int keep_set1)
 {
+    chain_start();
     h->err = kNoError;
     h->maxlen[0] = 0;
     if (!keep_set1) h->maxlen[1] = 0;
@@ -48,7 +49,11 @@ __global__ void init_header_kernel(Header* h, int keep_set1)
 
 // The persistent walks take work units from h->tiles upward; starting the
 // counter at u0 makes a launch walk units u0 .. (its tile count) x units - 1.
-__global__ void reset_tiles_kernel(Header* h, unsigned long long u0) { h->tiles = u0; }
+__global__ void reset_tiles_kernel(Header* h, unsigned long long u0)
+{
+    chain_start();
+    h->tiles = u0;
+}
 
 // Rows of the FULL matrices whose pairs have all been written, copied from
 // the device matrices to page-locked host matrices (device-accessible
@@ -528,7 +533,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
             wa.p[k] = f.metric == PCF_LP ? f.p : (f.metric == PCF_L2 ? 2.0 : 1.0);
         }
         if (kernel != PCF_SCHED_MERGEPATH)
-            reset_tiles_kernel<<<1, 1, 0, s>>>(wa.hdr, (unsigned long long)unit0);
+            launch_next(reset_tiles_kernel, 1, 1, 0, s, wa.hdr, (unsigned long long)unit0);
         cudaError_t e;
         const int g = (int)grid;
         // launcher of (schedule, precision, form)
@@ -719,7 +724,7 @@ int pcf_prepare(const pcf_csr* x, int precision, void* workspace, size_t workspa
     int form = kPackF64;
     int rc = pairwise_common(x, precision, workspace, workspace_bytes, &hdr, &sv, &ks, &form);
     if (rc != PCF_OK) return rc;
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     if (x->n == 0) return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
     if (prepare_pairwise(x, form, hdr, sv, ks, stream, pr.auto64) != cudaSuccess) return PCF_ECUDA;
     return PCF_OK;
@@ -757,7 +762,7 @@ int pcf_pairwise_ex(const pcf_csr* x, const pcf_integral* F, int nF, int precisi
     if (rc != PCF_OK) return rc;
     if (x->n == 0) return PCF_OK;
     if (!(flags & PCF_PAIRWISE_PREPARED)) {
-        init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+        launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
         if (prepare_pairwise(x, form, hdr, sv, ks, stream, pr.auto64) != cudaSuccess) return PCF_ECUDA;
     }
 
@@ -823,7 +828,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
         vec16 = vec16 && (uintptr_t)cp.src[k] % 16 == 0 && (uintptr_t)cp.dst[k] % 16 == 0;
     }
 
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     if (prepare_pairwise(x, form, hdr, sv, ks, stream, pr.auto64) != cudaSuccess) return PCF_ECUDA;
     WalkArgs wa;
     memset(&wa, 0, sizeof wa);
@@ -993,7 +998,7 @@ static int cross_impl(const pcf_csr* a, const pcf_csr* b, int64_t row_begin, int
     KeySort ks;
     if (form == kPackKeyed) ks = carve_keysort(cur, key_capacity(a, b));
     const bool reuse = (flags & PCF_CROSS_REUSE_B) != 0;
-    if (!moved) init_header_kernel<<<1, 1, 0, stream>>>(hdr, reuse ? 1 : 0);
+    if (!moved) launch_next(init_header_kernel, 1, 1, 0, stream, hdr, reuse ? 1 : 0);
     // keyed: B's interval ends first in the sort input, then A's; both are
     // ranked together every call (A's rows change, so B's ranks do too: a
     // reused B keeps its validation and length sort and is packed again)
@@ -1131,7 +1136,7 @@ int pcf_pairwise_backward_ex(const pcf_csr* x, int metric, double p, int apply_r
     double* gv = (double*)cur;
     cur += align_up(sizeof(double) * (size_t)x->nnz);
     double* gt = (double*)cur;
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     if (prepare_set(x->offsets, x->times, x->values, x->dtype, x->n, x->nnz, true, kPackF64, hdr,
                     sv, stream) != cudaSuccess)
         return PCF_ECUDA;
@@ -1175,7 +1180,7 @@ int pcf_segment_integrals(const pcf_csr* x, int functional, double p, int apply_
     SetView sv;
     int rc = pairwise_common(x, PCF_PREC_F64, workspace, workspace_bytes, &hdr, &sv);
     if (rc != PCF_OK) return rc;
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     if (x->n == 0) return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
     // the input check runs inside the segment kernels (same reasons and indices)
     // scratch in the packed area: the chunk table and the long-PCF pieces
@@ -1289,7 +1294,7 @@ int pcf_pairwise_weighted(const pcf_csr* x, const pcf_csr* w, const pcf_integral
     rc = pairwise_common(&m, precision, workspace, inner, &hdr, &sv, &ks, &form);
     if (rc != PCF_OK) return rc;
 
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     // x and w are checked before the moved collection is built from them
     if (launch_validate(x->offsets, x->times, x->values, x->dtype, x->n, x->nnz, kPackF64, hdr, sv,
                         stream) != cudaSuccess ||
@@ -1395,7 +1400,7 @@ int pcf_cross_weighted(const pcf_csr* a, const pcf_csr* b, int64_t row_begin, in
     if (form == kPackKeyed && key_capacity(&am, &bm) > 0x7fffffffLL) return PCF_EUNSUPPORTED;
 
     Header* hdr = (Header*)workspace;
-    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
+    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
     // the inputs are checked before they are moved (scratch set views of the
     // cross workspace serve the checks' length arrays)
     {

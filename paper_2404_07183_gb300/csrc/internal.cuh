@@ -228,6 +228,39 @@ struct KeyOut {
 size_t set_bytes(int64_t n, int64_t nnz, int elem_bytes);
 SetView carve_set(char*& cursor, int64_t n, int64_t nnz, int elem_bytes, int slot);
 
+// Kernels of a call follow one another at once: each is launched as a
+// programmatic dependent of the one before (launch_next) and waits for it to
+// complete (and for what it waited for) before it touches memory; the short
+// kernels of the preparation let their successor be placed as soon as all
+// their own CTAs run (chain_start), so that its launch does not add to the
+// chain.  The walks only wait: a successor placed beside them would hold
+// resources for their whole time.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_start()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_wait();
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s,
+                        A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Validate + sort + pack one collection given by absolute CSR offsets

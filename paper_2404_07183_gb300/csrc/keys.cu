@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(256) count_keys_kernel(Header* hdr, const int6
                                                          const int64_t* poff1, int64_t n1,
                                                          uint32_t* __restrict__ misc)
 {
+    chain_start();
     for (int i = threadIdx.x; i < kMiscWords; i += 256) misc[i] = 0;
     if (threadIdx.x != 0) return;
     // no keys after an input error, or when an AUTO64 call walks in float64
@@ -173,6 +174,7 @@ radix_hist_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ misc,
     __shared__ int last, trivial[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t gid = (int64_t)blockIdx.x * 256 + tid, gsz = (int64_t)gridDim.x * 256;
+    chain_start();
     for (int64_t i = gid; i < nstatus; i += gsz) status[i] = 0;
     for (int64_t i = gid; i < ntsum; i += gsz) tsum[i] = 0;
     for (int d = 0; d < 8; ++d) cnt[d][tid] = 0;
@@ -265,6 +267,7 @@ radix_pass_kernel(uint64_t* __restrict__ key0, uint64_t* __restrict__ key1, uint
     __shared__ uint32_t wsum[8];
     __shared__ int64_t s_tile;
     __shared__ int s_fail;
+    chain_start();
     const uint32_t plan = misc[kMiscPlan + pass];
     if (plan > 1u) return;                                  // all keys share this digit
     const uint64_t* kin = plan ? key1 : key0;
@@ -378,6 +381,7 @@ rank_write_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict_
     __shared__ int64_t s_tile;
     __shared__ int s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_start();
     const bool one = misc[kMiscFinal] != 0u;
     const uint64_t* key = one ? key1 : key0;
     const uint32_t* pay = one ? pay1 : pay0;
@@ -441,6 +445,7 @@ __global__ void bound_keys_kernel(const uint64_t* __restrict__ key0, const uint6
                                   const uint32_t* __restrict__ misc, const KElem* pack0, const KElem* pack1, double a, double b,
                                   Header* hdr)
 {
+    chain_start();
     const int64_t m = (int64_t)hdr->nkeys;
     const uint64_t* key = misc[kMiscFinal] ? key1 : key0;
     const uint32_t* pay = misc[kMiscFinal] ? pay1 : pay0;
@@ -466,7 +471,7 @@ __global__ void bound_keys_kernel(const uint64_t* __restrict__ key0, const uint6
 cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int64_t n0,
                       KElem* pack1, const int64_t* poff1, int64_t n1, Header* hdr, cudaStream_t s)
 {
-    count_keys_kernel<<<1, 256, 0, s>>>(hdr, poff0, n0, poff1, n1, ks.misc);
+    launch_next(count_keys_kernel, 1, 256, 0, s, hdr, poff0, n0, poff1, n1, ks.misc);
     const unsigned tiles = (unsigned)ks.tiles;
     const int wide = ks.cap >= kNarrowKeys ? 1 : 0;
     cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -477,17 +482,17 @@ cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int
     const int64_t hcap = (int64_t)device_sm_count() * 4;
     if (hgrid > hcap) hgrid = hcap;
     if (hgrid < 1) hgrid = 1;
-    radix_hist_kernel<<<(unsigned)hgrid, 256, 0, s>>>(ks.key[0], ks.misc, ks.status, ks.tiles * 256,
+    launch_next(radix_hist_kernel, hgrid, 256, 0, s, ks.key[0], ks.misc, ks.status, ks.tiles * 256,
                                                       ks.tsum, ks.tiles + 1, hdr);
     for (int pass = 0; pass < 8; ++pass) {
         if (wide && pass > 0) {
             e = cudaMemsetAsync(ks.status, 0, sizeof(uint32_t) * 256 * (size_t)ks.tiles, s);
             if (e != cudaSuccess) return e;
         }
-        radix_pass_kernel<<<tiles, kSortThreads2, radix_pass_smem(), s>>>(
+        launch_next(radix_pass_kernel, tiles, kSortThreads2, radix_pass_smem(), s,
             ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.status, ks.misc, pass, wide, hdr);
     }
-    rank_write_kernel<<<tiles, kSortThreads2, 0, s>>>(ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.tsum,
+    launch_next(rank_write_kernel, tiles, kSortThreads2, 0, s, ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.tsum,
                                                       ks.misc, pack0, pack1, hdr);
     return cudaGetLastError();
 }
@@ -495,7 +500,7 @@ cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int
 cudaError_t bound_keys(const KeySort& ks, const KElem* pack0, const KElem* pack1, double a, double b,
                        Header* hdr, cudaStream_t s)
 {
-    bound_keys_kernel<<<1, 1, 0, s>>>(ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.misc, pack0, pack1, a, b, hdr);
+    launch_next(bound_keys_kernel, 1, 1, 0, s, ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.misc, pack0, pack1, a, b, hdr);
     return cudaGetLastError();
 }
 

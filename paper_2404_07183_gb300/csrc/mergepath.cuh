@@ -284,6 +284,8 @@ cudaError_t launch_mergepath_t(int combo, const WalkArgs& a, int64_t npairs, int
     const int64_t sms = device_sm_count();
     const int64_t mine = (npairs - a.shard_index + a.shard_count - 1) / a.shard_count;
     if (mine < 1) return cudaSuccess;
+    // (not launched by launch_next: clusters placed before the pack has left
+    // its SMs end up unevenly spread, 25 long curves 216 -> 231 us per call)
     auto go = [&](auto kern, int64_t grid, int parts, size_t smem) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

@@ -32,6 +32,7 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
                                 int32_t* __restrict__ lens, uint32_t* __restrict__ skey,
                                 Header* hdr, int slot, int auto64, int skip_on_error, int fs)
 {
+    chain_start();
     // a collection built by an earlier kernel of the call is only checked
     // when that kernel ran (no error recorded before it)
     if (skip_on_error && hdr->err != kNoError) return;
@@ -128,6 +129,7 @@ sort_scan_kernel(const int32_t* __restrict__ lens, const uint32_t* __restrict__ 
     __shared__ int64_t carry_s;
     __shared__ int64_t warp_sums[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    chain_start();
     if (hdr->err != kNoError) return;
 
     const unsigned int maxlen = hdr->maxlen[slot];
@@ -269,6 +271,7 @@ sort_small_kernel(const int32_t* __restrict__ lens, const uint32_t* __restrict__
     __shared__ int32_t xi[kSortSmall];
     __shared__ int64_t wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, P = blockDim.x;
+    chain_start();
     if (hdr->err != kNoError) return;
     const bool use_scale = hdr->maxlen[slot] > (unsigned)kScaleSortMin;
     unsigned long long k = ~0ull;                  // past the end: after every PCF
@@ -333,6 +336,7 @@ __global__ void pack_kernel(const int64_t* __restrict__ offsets, const Tin* __re
                             const unsigned int* gate, int want64, int fs)
 {
     using E = typename Elem<Tin, Tw>::type;
+    chain_start();
     if (hdr->err != kNoError || gated_off(gate, want64)) return;
     E* packed = reinterpret_cast<E*>(packed_v);
     const int lane = threadIdx.x & 31;
@@ -370,6 +374,7 @@ __global__ void pack_keyed_kernel(const int64_t* __restrict__ offsets,
                                   KElem* __restrict__ packed, KeyOut ko, const Header* hdr,
                                   const unsigned int* gate, int want64, int fs)
 {
+    chain_start();
     if (hdr->err != kNoError || gated_off(gate, want64)) return;
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -461,11 +466,11 @@ cudaError_t launch_validate(const int64_t* offsets, const void* times, const voi
     const int g = grid_for_warps(n << fs);
     const int walk_f32 = form != kPackF64;
     if (in_dtype == PCF_F64) {
-        validate_kernel<double><<<g, 256, 0, s>>>(offsets, (const double*)times,
+        launch_next(validate_kernel<double>, g, 256, 0, s, offsets, (const double*)times,
             (const double*)values, n, nnz_total, whole, walk_f32, sv.lens, sv.skey, hdr, sv.slot, 0, 0,
             fs);
     } else {
-        validate_kernel<float><<<g, 256, 0, s>>>(offsets, (const float*)times,
+        launch_next(validate_kernel<float>, g, 256, 0, s, offsets, (const float*)times,
             (const float*)values, n, nnz_total, whole, walk_f32, sv.lens, sv.skey, hdr, sv.slot, 0, 0,
             fs);
     }
@@ -482,29 +487,29 @@ cudaError_t pack_set(const int64_t* offsets, const void* times, const void* valu
     if (form == kPackKeyed) {
         if (!ko) return cudaErrorInvalidValue;
         if (in_dtype == PCF_F64)
-            pack_keyed_kernel<double><<<g, 256, 0, s>>>(offsets, (const double*)times,
+            launch_next(pack_keyed_kernel<double>, g, 256, 0, s, offsets, (const double*)times,
                 (const double*)values, n, sv.perm, sv.slen, sv.poff,
                 reinterpret_cast<KElem*>(sv.packed), *ko, hdr, gate, want64, fs);
         else
-            pack_keyed_kernel<float><<<g, 256, 0, s>>>(offsets, (const float*)times,
+            launch_next(pack_keyed_kernel<float>, g, 256, 0, s, offsets, (const float*)times,
                 (const float*)values, n, sv.perm, sv.slen, sv.poff,
                 reinterpret_cast<KElem*>(sv.packed), *ko, hdr, gate, want64, fs);
     } else if (in_dtype == PCF_F64) {
         if (form == kPackF64)
-            pack_kernel<double, double><<<g, 256, 0, s>>>(offsets, (const double*)times,
+            launch_next(pack_kernel<double, double>, g, 256, 0, s, offsets, (const double*)times,
                 (const double*)values, n, sv.perm, sv.slen, sv.poff, sv.packed, hdr, gate, want64,
                 fs);
         else
-            pack_kernel<double, float><<<g, 256, 0, s>>>(offsets, (const double*)times,
+            launch_next(pack_kernel<double, float>, g, 256, 0, s, offsets, (const double*)times,
                 (const double*)values, n, sv.perm, sv.slen, sv.poff, sv.packed, hdr, gate, want64,
                 fs);
     } else {
         if (form == kPackF64)
-            pack_kernel<float, double><<<g, 256, 0, s>>>(offsets, (const float*)times,
+            launch_next(pack_kernel<float, double>, g, 256, 0, s, offsets, (const float*)times,
                 (const float*)values, n, sv.perm, sv.slen, sv.poff, sv.packed, hdr, gate, want64,
                 fs);
         else
-            pack_kernel<float, float><<<g, 256, 0, s>>>(offsets, (const float*)times,
+            launch_next(pack_kernel<float, float>, g, 256, 0, s, offsets, (const float*)times,
                 (const float*)values, n, sv.perm, sv.slen, sv.poff, sv.packed, hdr, gate, want64,
                 fs);
     }
@@ -522,21 +527,21 @@ cudaError_t prepare_set(const int64_t* offsets, const void* times, const void* v
     const int walk_f32 = form != kPackF64;
     const int a64 = auto64 && walk_f32 ? 1 : 0;
     if (in_dtype == PCF_F64) {
-        validate_kernel<double><<<g, 256, 0, s>>>(offsets, (const double*)times,
+        launch_next(validate_kernel<double>, g, 256, 0, s, offsets, (const double*)times,
             (const double*)values, n, nnz_total, whole, walk_f32, sv.lens, sv.skey, hdr, sv.slot,
             a64, built ? 1 : 0, fs);
     } else {
-        validate_kernel<float><<<g, 256, 0, s>>>(offsets, (const float*)times,
+        launch_next(validate_kernel<float>, g, 256, 0, s, offsets, (const float*)times,
             (const float*)values, n, nnz_total, whole, walk_f32, sv.lens, sv.skey, hdr, sv.slot,
             a64, built ? 1 : 0, fs);
     }
     if (n <= kSortSmall) {
         int threads = 32;
         while (threads < n) threads <<= 1;
-        sort_small_kernel<<<1, threads, 0, s>>>(sv.lens, sv.skey, (int)n, hdr, sv.slot, sv.perm, sv.slen,
+        launch_next(sort_small_kernel, 1, threads, 0, s, sv.lens, sv.skey, (int)n, hdr, sv.slot, sv.perm, sv.slen,
                                                 sv.poff);
     } else {
-        sort_scan_kernel<<<1, kSortThreads, 0, s>>>(sv.lens, sv.skey, n, hdr, sv.slot, sv.perm, sv.slen,
+        launch_next(sort_scan_kernel, 1, kSortThreads, 0, s, sv.lens, sv.skey, n, hdr, sv.slot, sv.perm, sv.slen,
                                                     sv.khi[0], sv.klo[0], sv.kv[0], sv.khi[1], sv.klo[1],
                                                     sv.kv[1], sv.poff);
     }

@@ -477,6 +477,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     __shared__ int64_t sUnit;
     __shared__ int64_t sBlock[2];                   // the unit's row and column block
 
+    chain_wait();
     if (gated_off(a.gate, a.gate_want64)) return;   // the other walk of an AUTO64 call
     if (block_sees_error(a.hdr)) return;
 
@@ -957,8 +958,7 @@ cudaError_t launch_walk_tt(int combo, const WalkArgs& a, int grid, size_t smem, 
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<grid, THREADS, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_next(kern, grid, THREADS, smem, s, a);
     };
     switch (combo) {
     case kComboL1: return go(walk_kernel<T, PREC, kComboL1, THREADS, CTAS, WEIGHT, KEYED>);
