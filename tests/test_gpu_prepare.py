@@ -82,3 +82,32 @@ def test_errors_of_split_validation(pcf, n, length):
     with pytest.raises(pcf.PcfError) as e:
         pcf.pcf_pairwise(x, ["l1"])
     assert (e.value.detail, e.value.index) == (3, k)
+
+
+@pytest.mark.parametrize("prec,dtype", [("f64", np.float64), ("f32c", np.float64), ("f64", np.float32)])
+@pytest.mark.parametrize("bad,detail", [
+    ([-0.0, -0.0], 3), ([-0.0, 0.0], 3), ([0.0, -0.0], 3), ([0.0, -1.0], 3), ([-1.0, -0.5], 2),
+    ([0.0, 1.0, 1.0], 3), ([0.0, np.nan, 1.0], 4), ([0.0, np.inf], 4), ([0.0, -np.inf, 2.0], 4),
+    ([5e-324, 1.0], 2), ([0.0, 2.0, 1.0, 3.0], 3)], ids=str)
+def test_time_checks(pcf, bad, detail, prec, dtype):
+    """Zeros of either sign, negative and non-finite times: reason and index."""
+    t = np.concatenate([[0.0, 1.0], bad, [0.0, 3.0]])
+    o = np.array([0, 2, 2 + len(bad), 4 + len(bad)])
+    x = pcf.PcfTensors.from_numpy(synth.PcfSet(o, t.astype(dtype), np.zeros(t.size, dtype)), "cuda")
+    if dtype == np.float32 and bad[0] == 5e-324:
+        return                                       # 0 in float32
+    k = 2 if detail == 2 else 2 + next(
+        i for i in range(1, len(bad)) if not (np.isfinite(bad[i]) and bad[i] > bad[i - 1]))
+    with pytest.raises(pcf.PcfError) as e:
+        pcf.pcf_pairwise(x, ["l1"], precision=prec)
+    assert (e.value.detail, e.value.index) == (detail, k)
+
+
+@pytest.mark.parametrize("t", [[-0.0, 1.0, 2.0], [-0.0], [0.0, 5e-324, 1e-310]], ids=str)
+def test_times_that_pass(pcf, t):
+    import torch
+    s = synth.PcfSet([0, 1, 1 + len(t)], np.concatenate([[0.0], t]),
+                     np.concatenate([[0.0], np.arange(len(t), dtype=float)[::-1]]))
+    got = pcf.pcf_pairwise(pcf.PcfTensors.from_numpy(s, "cuda"), ["l1"], precision="f64",
+                           out_dtype=torch.float64)[0].cpu().numpy()
+    np.testing.assert_array_equal(got, oracle.matrix(s, metric="l1"))
