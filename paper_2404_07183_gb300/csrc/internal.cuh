@@ -22,6 +22,7 @@
 
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <utility>
 
 #include "../../include/pcf.h"
 
@@ -243,9 +244,10 @@ __device__ __forceinline__ void chain_start()
     chain_wait();
 }
 
+// at_once = false: an ordinary launch.
 template <typename... P, typename... A>
-cudaError_t launch_next(void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s,
-                        A&&... args)
+cudaError_t launch_kernel(bool at_once, void (*kernel)(P...), int64_t grid, int threads, size_t smem,
+                          cudaStream_t s, A&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -256,8 +258,15 @@ cudaError_t launch_next(void (*kernel)(P...), int64_t grid, int threads, size_t 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = at_once ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s,
+                        A&&... args)
+{
+    return launch_kernel(true, kernel, grid, threads, smem, s, std::forward<A>(args)...);
 }
 #endif
 
@@ -296,6 +305,8 @@ struct WalkArgs {
     int tile_order;          // symmetric tile order: 0 = column blocks from the last
                              // down, 1 = row blocks from the first up (each with its
                              // longest partner first)
+    int at_once;             // 1: walks launched as programmatic dependents; 0: in the
+                             // ordinary way (bands whose copies run beside the next walk)
     int window;              // W: staged elements per PCF per window
     Header* hdr;
     // outputs

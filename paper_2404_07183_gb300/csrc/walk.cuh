@@ -958,7 +958,7 @@ cudaError_t launch_walk_tt(int combo, const WalkArgs& a, int grid, size_t smem, 
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        return launch_next(kern, grid, THREADS, smem, s, a);
+        return launch_kernel(a.at_once != 0, kern, grid, THREADS, smem, s, a);
     };
     switch (combo) {
     case kComboL1: return go(walk_kernel<T, PREC, kComboL1, THREADS, CTAS, WEIGHT, KEYED>);
