@@ -93,7 +93,9 @@ enum pcf_precision {
  * rounded to float32
  * (the walk's arithmetic).  Such a call needs nnz (both collections together
  * for a cross call) below 2^31, else PCF_EUNSUPPORTED.  The p-th root is
- * always taken in float64.
+ * taken in float64; for float32 outputs of a float32 walk the square and cube
+ * roots are float32 roots with a correction step, good to about 2^-44 before
+ * the one rounding to float32.
  *
  * PCF_PREC_ROUND_TIMES, or-ed into a float32 precision, asks for the faster
  * packed form instead: float64 times rounded to nearest float32 when packed
@@ -162,8 +164,10 @@ enum pcf_cross_flags {
  *   PCF_SCHED_AUTO        merge path for few pairs (14,000 for float32 walks,
  *                         45,000 for float64), else TILE_512X3 for float32
  *                         walks of float32 input with one metric but general
- *                         p, TILE_512X2 for the others, and TILE_1024 for
- *                         rounded times, an explicit window or lambda > 0 */
+ *                         p, TILE_512X2 for the others, TILE_1024 for
+ *                         lambda > 0.  With rounded times or an explicit
+ *                         window: merge path when there are fewer tiles than
+ *                         half the SMs, else TILE_1024 */
 enum pcf_sched_kernel {
     PCF_SCHED_AUTO = 0, PCF_SCHED_TILE_1024 = 1, PCF_SCHED_TILE_512X2 = 2,
     PCF_SCHED_MERGEPATH = 3, PCF_SCHED_TILE_512X3 = 4

@@ -424,13 +424,12 @@ int check_window(const pcf_window* w)
 // metrics 20.8 / 19.2 / 19.8; float64 N = 1,000 0.461 / 0.407 / 0.414.  Two
 // CTAs let one issue while the other waits at a tile barrier.  The third pays
 // where 40 registers hold the walk: 8-byte elements and one metric without
-// pow.  TILE_1024 stays where its larger window decides what is accepted
-// (rounded times: coincident times must fit one window; an explicit window)
-// and for the exp(-lambda t) weights, which only it has.
-int auto_tile_kernel(const pcf_integral* F, int nF, int form, bool round, bool weighted,
-                     bool explicit_window)
+// pow.  TILE_1024 stays for the exp(-lambda t) weights, which only it has, and
+// (auto_kernel) where its larger window decides what is accepted: rounded
+// times, whose coincident times must fit one window, and explicit windows.
+int auto_tile_kernel(const pcf_integral* F, int nF, int form, bool weighted)
 {
-    if (weighted || round || explicit_window) return PCF_SCHED_TILE_1024;
+    if (weighted) return PCF_SCHED_TILE_1024;
     if (form != kPackF32) return PCF_SCHED_TILE_512X2;
     for (const Launch& L : plan(F, nF))
         if (L.n > 1 || L.combo == kComboLP) return PCF_SCHED_TILE_512X2;
@@ -450,10 +449,16 @@ constexpr int64_t kMpPairsF32 = 14000, kMpPairsF64 = 45000;
 int auto_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool round,
                 bool windowed, bool weighted, const pcf_schedule* sched)
 {
+    // what a call with rounded times or an explicit window accepts depends on
+    // the kernel (the merge path has no window to overflow): fewer tiles than
+    // half the SMs go to the merge path there, as ever
+    if (round || (sched && sched->window != 0))
+        return wa.ntiles * 2 < device_sm_count() && !windowed ? PCF_SCHED_MERGEPATH
+                                                              : PCF_SCHED_TILE_1024;
     const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
     if (!windowed && pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32))
         return PCF_SCHED_MERGEPATH;
-    return auto_tile_kernel(F, nF, form, round, weighted, sched && sched->window != 0);
+    return auto_tile_kernel(F, nF, form, weighted);
 }
 
 bool is_windowed(const pcf_window* w)

@@ -63,3 +63,39 @@ def test_dyadic_bitwise(pcf, lens):
             if prec == "f32c" and max(lens) > 1000:
                 continue                                # sums beyond 2^24
             np.testing.assert_array_equal(g.cpu().numpy(), oracle.matrix(s, metric=m))
+
+
+@pytest.mark.parametrize("lens", [[300, 213, 43], [20000, 16385, 12001]], ids=str)
+def test_captured_call(pcf, lens):
+    """A captured call (plain and cluster launches) replays with new contents."""
+    import torch
+    sets = [synth.from_lengths(lens, lambda r, m: r.exponential(1.0, m),
+                               lambda r, o: np.where(np.isin(np.arange(o[-1]), o[1:] - 1), 0.0,
+                                                     r.standard_normal(o[-1])),
+                               np.random.default_rng(seed), np.float64) for seed in (1, 2)]
+    x = pcf.PcfTensors.from_numpy(sets[0], "cuda")
+    for prec in ("f64", "f32c"):
+        graph = pcf.PairwiseGraph(x, ["l1"], precision=prec, out_dtype=torch.float64)
+        y = pcf.PcfTensors.from_numpy(sets[1], "cuda")
+        x.times.copy_(y.times)
+        x.values.copy_(y.values)
+        got = graph.replay()[0].clone()
+        graph.check()
+        want = pcf.pcf_pairwise(y, ["l1"], precision=prec, out_dtype=torch.float64)[0]
+        assert torch.equal(got, want)
+
+
+def test_auto_keeps_what_windows_and_rounding_accept(pcf):
+    """200 PCFs (fewer tiles than half the SMs): an explicit window larger than any
+    tile kernel's, and rounded times with more coincident ones than a window holds,
+    go to the merge path."""
+    import torch
+    s = synth.random_set(200, seed=3, min_len=5, max_len=30)
+    x = pcf.PcfTensors.from_numpy(s, "cuda")
+    got = pcf.pcf_pairwise(x, ["l1"], precision="f32c", schedule=("auto", 4000), out_dtype=torch.float64)[0]
+    assert max_rel_error("l1", got.cpu().numpy(), oracle.matrix(s, metric="l1")) <= 1e-5
+    t = np.concatenate([[0.0], 4096.0 + 2.0 ** -20 * np.arange(1, 600)])
+    o = np.arange(0, 200 * t.size + 1, t.size)
+    v = np.tile(np.concatenate([np.arange(t.size - 1) % 7, [0.0]]), 200)
+    pcf.pcf_pairwise(pcf.PcfTensors.from_numpy(synth.PcfSet(o, np.tile(t, 200), v), "cuda"), ["l1"],
+                     precision="f32c_round")
