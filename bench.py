@@ -59,13 +59,23 @@ def tally(prec, input_f64=True):
     """Operations per merge step of the walk a precision name runs on this input."""
     keyed = input_f64 and prec in ("f32c", "f32b", "f32")
     return TALLY[prec] + (KEYED_EXTRA if keyed else 0)
-FP64_OPS_PER_STEP = 1 + 1 + 1 + 2 + 2   # dt, d, L1 fma, L2 mul+fma, Gram mul+fma
+
+
+def fp64_ops(metrics, schedule):
+    """Operations per merge step on the float64 pipe: the accumulation of each
+    metric and the difference of L1 and L2.  The width dt and the products of
+    L2 and Gram run on the integer pipes, except with three CTAs per SM and on
+    the merge path."""
+    n = len(metrics) + (1 if set(metrics) & {"l1", "l2"} else 0)
+    if schedule in ("tile512x3", "mergepath"):
+        n += 1 + len(set(metrics) & {"l2", "gram"})
+    return n
 
 # DRAM bytes (read + write) per launch of the benchmark's compensated walk,
 # from one ncu capture (profiles/walk_f32ck_dram_traffic_stable_rank_n20000.md),
 # valid only while the walk's source is the one that was measured.
-TRAFFIC_RECORD = {"source_sha256_16": "cc8a5afd078a05bc+cbd8c1c574e4db57",
-                  "by_schedule_layout": {("tile512x2", "full"): 1206109440 + 4928763392}}
+TRAFFIC_RECORD = {"source_sha256_16": "edd8e1ec5b550ed1+4091e163e9ee196c",
+                  "by_schedule_layout": {("tile512x2", "full"): 1192259584 + 4747656192}}
 
 
 def walk_source_id():
@@ -87,11 +97,11 @@ def dist_env():
 def step_launches(prec, layout="full", input_f64=True):
     """Kernels one timed step launches: pcf_prepare (header, validation,
     length sort, pack; for float64 input in a float32 walk the key sort: key
-    count, 8 passes of histogram + two row scans + scatter, distinct-key
-    count, its scan and the rank write), pcf_pairwise (tile counter, walk;
-    FULL layout: inverse permutation and the column pass)."""
+    count, digit counts of all passes, 8 passes, rank write), pcf_pairwise
+    (tile counter, walk; FULL layout: inverse permutation and the column
+    pass)."""
     keyed = input_f64 and prec in ("f32c", "f32b", "f32")
-    n = 4 + (1 + 8 * 4 + 3 if keyed else 0) + 2
+    n = 4 + (2 + 8 + 1 if keyed else 0) + 2
     return n + (2 if layout == "full" else 0)
 
 
@@ -597,9 +607,10 @@ def run_ours(args):
             basis = f"tally {tally(name)} ops per merge step"
         else:
             r64 = pp["fp64"]["lane_ops_per_clk_per_sm"]
-            pk = sms * r64 * fmax / FP64_OPS_PER_STEP
+            ops = fp64_ops(METRICS, f["schedule"])
+            pk = sms * r64 * fmax / ops
             basis = (f"{sms} SMs x {r64:.2f} FP64 lane-ops/clk x {fmax/1e6:.0f} MHz / "
-                     f"{FP64_OPS_PER_STEP} FP64 ops per step")
+                     f"{ops} ops per step on the FP64 pipe")
         d = {"value": units * pairs / (f["ms_per_step"] * 1e-3), "unit": "pair-integrals/s",
              "ms_per_step": f["ms_per_step"], "walk_ms": f["walk_ms"], "prepare_ms": f["prepare_ms"],
              "merge_steps_per_s": wr, "schedule": f["schedule"],
@@ -791,6 +802,7 @@ def run_workload(name, args):
             P.pcf_check(ws)
             out[prec] = float(np.mean(ms))
         ms = out["f64"]
+        l1_ops = fp64_ops(["l1"], tuned["f64"]["schedule"])
         rate = steps_walk / (ms * 1e-3)
         return _line(name, pairs / (ms * 1e-3), "pair-integrals/s", ms, args.steps, args.warmup,
                      "f64", {"workload": "uniform_small N=1000 n~U{10..100} Exp(1) N(0,1) "
@@ -798,8 +810,8 @@ def run_workload(name, args):
                              "merge_steps": steps_walk, "cuda_graph": True,
                              "l2": "flushed between steps", "autotune": tuned},
                      merge_steps_per_s=rate,
-                     roofline={"bound": "fp64 pipe", "achieved": rate, "peak": fp64(3),
-                               "unit": "merge-steps/s", "frac": rate / fp64(3),
+                     roofline={"bound": "fp64 pipe", "achieved": rate, "peak": fp64(l1_ops),
+                               "unit": "merge-steps/s", "frac": rate / fp64(l1_ops),
                                "note": "whole step (prepare + walk, 6 launches in one graph)"},
                      f32c={"ms_per_step": out["f32c"], "value": pairs / (out["f32c"] * 1e-3)},
                      cpu_baseline=_cpu_rows(s, ["l1"], seconds_target=4.0))
@@ -844,8 +856,7 @@ def run_workload(name, args):
             res[prec] = float(np.mean(ms))
             del ws
         ms = res["f32c"]
-        # float64 operations per merge step of the Gram walk: dt, a*b, fma
-        gram64_ops = 3
+        gram64_ops = fp64_ops(["gram"], scheds["f64"])
         rate = (steps_walk + diag) / (ms * 1e-3)
         tally = 5 + 2 + 3
         return _line(name, pairs / (ms * 1e-3), "pair-integrals/s", ms, max(1, min(args.steps, 2)),
@@ -865,7 +876,7 @@ def run_workload(name, args):
                            "merge_steps_per_s": (steps_walk + diag) / (res["f64"] * 1e-3),
                            "frac": (steps_walk + diag) / (res["f64"] * 1e-3) / fp64(gram64_ops),
                            "bound": "fp64 pipe", "schedule": scheds["f64"],
-                           "note": f"{gram64_ops} float64 ops per merge step (dt, a*b, fma); "
+                           "note": f"{gram64_ops} operations per merge step on the float64 pipe; "
                                    "one timed step"},
                      cpu_baseline=(None if args.no_cpu else
                                    _cpu_rows(s, ["gram"], seconds_target=8.0, row0=N // 2)))
@@ -946,6 +957,7 @@ def run_workload(name, args):
         rate = (steps_walk + diag_steps) / (ms * 1e-3)
         tally = TALLY["f32c"] + KEYED_EXTRA
         r64 = (steps_walk + diag_steps) / (res["f64"]["ms_per_step"] * 1e-3)
+        f64_ops = fp64_ops(METRICS, res["f64"]["schedule"])
         cpu = _cpu_rows_weighted(s, (tw, vw), seconds_target=8.0)
         return _line(name, pairs / (ms * 1e-3), "pair-integrals/s", ms,
                      max(1, min(args.steps, 3)), 1, "f32 (compensated)",
@@ -963,8 +975,8 @@ def run_workload(name, args):
                      fp64={"value": pairs / (res["f64"]["ms_per_step"] * 1e-3),
                            "ms_per_step": res["f64"]["ms_per_step"], "merge_steps_per_s": r64,
                            "roofline": {"bound": "fp64 pipe", "achieved": r64,
-                                        "peak": fp64(FP64_OPS_PER_STEP),
-                                        "frac": r64 / fp64(FP64_OPS_PER_STEP)}},
+                                        "peak": fp64(f64_ops),
+                                        "frac": r64 / fp64(f64_ops)}},
                      forms=res, cpu_baseline=cpu)
 
     if name == "segments":
@@ -1129,10 +1141,11 @@ def run_workload(name, args):
         if not args.no_cpu and rank == 0:
             oracle.backward(sub, G[:300, :300], metric="l2", p=2.0)
         dt = max(time.perf_counter() - t0, 1e-9)
-        # float64 operations per rectangle of the L2 adjoint: dt, d, d*dt, two
-        # value-gradient fma; time gradient of the advancing side: v_new - v_other,
-        # its square, fma(d, d, -b*b), times the weight
-        bw_ops = 9
+        # operations per rectangle that the L2 adjoint leaves on the float64 pipe:
+        # d*dt, two value-gradient sums, v_new - v_other, and two for the time
+        # gradient of the advancing side (d is carried on, widths and squares run
+        # on the integer pipes)
+        bw_ops = 6
         cfg = {"workload": "gradient N=4096 n~U{20..200} Exp(1) N(0,1) float64, "
                            "d(sum G*D2^2)/d(values, times)", "N": N, "pairs": pairs,
                "merge_steps": steps_walk, "l2": "flushed between steps"}
@@ -1147,7 +1160,7 @@ def run_workload(name, args):
                                "unit": "merge-steps/s", "frac": rate / (fp64(bw_ops) * world),
                                "note": f"whole backward call (recomputing walk + scatter"
                                        f"{' + all-reduce' if world > 1 else ''}); "
-                                       f"{bw_ops} float64 ops per merge step"
+                                       f"{bw_ops} operations per merge step on the float64 pipe"
                                        f"{f', peak of {world} GPUs' if world > 1 else ''}"},
                      **extra,
                      cpu_baseline={"value": 300 * 299 / 2 / dt, "unit": "pair-gradients/s",

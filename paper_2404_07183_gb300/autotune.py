@@ -3,8 +3,9 @@
 For a class of inputs (GPU, precision, metric set, layout, and the binned
 size N, mean and maximum PCF length), it times every candidate schedule of
 ``pcf_pairwise_ex`` on the actual collection -- 32 x 32 tiles with one
-1024-thread CTA per SM, the same tiles with two 512-thread CTAs per SM, and
-the warp-per-pair merge path -- and remembers the fastest in a JSON cache
+1024-thread CTA per SM, the same tiles with two or three 512-thread CTAs per
+SM, and the merge path (a warp, a CTA or a cluster per pair) -- and remembers
+the fastest in a JSON cache
 (``$PCF_GB300_TUNE_CACHE`` or ``~/.cache/pcf_gb300/tune.json``).  Later
 calls in the same class use the cached schedule without timing again.
 """
