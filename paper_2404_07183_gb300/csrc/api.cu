@@ -1194,7 +1194,8 @@ int pcf_segment_integrals(const pcf_csr* x, int functional, double p, int apply_
     SetView sv;
     int rc = pairwise_common(x, PCF_PREC_F64, workspace, workspace_bytes, &hdr, &sv);
     if (rc != PCF_OK) return rc;
-    launch_next(init_header_kernel, 1, 1, 0, stream, hdr, 0);
+    // an ordinary launch: the segment kernels are not programmatic dependents
+    init_header_kernel<<<1, 1, 0, stream>>>(hdr, 0);
     if (x->n == 0) return cudaGetLastError() == cudaSuccess ? PCF_OK : PCF_ECUDA;
     // the input check runs inside the segment kernels (same reasons and indices)
     // scratch in the packed area: the chunk table and the long-PCF pieces
