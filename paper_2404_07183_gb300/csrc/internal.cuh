@@ -236,6 +236,13 @@ SetView carve_set(char*& cursor, int64_t n, int64_t nnz, int elem_bytes, int slo
 // their own CTAs run (chain_start), so that its launch does not add to the
 // chain.  The walks only wait: a successor placed beside them would hold
 // resources for their whole time.
+//
+// A kernel that may so be resident while earlier ones still write must read
+// what they write (and the caller's arrays, which the kernel before the call
+// may be writing) with ordinary coherent loads after its wait: no
+// `const __restrict__` parameters and no ld.global.nc, whose contract is that
+// the data does not change during the kernel, and which the compiler may move
+// across the wait.
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_start()

@@ -89,7 +89,7 @@ KeySort carve_keysort(char*& cur, int64_t cap)
 // from the packed offsets poff[n] of each set.  Clears the sort's counters.
 __global__ void __launch_bounds__(256) count_keys_kernel(Header* hdr, const int64_t* poff0, int64_t n0,
                                                          const int64_t* poff1, int64_t n1,
-                                                         uint32_t* __restrict__ misc)
+                                                         uint32_t* misc)
 {
     chain_start();
     for (int i = threadIdx.x; i < kMiscWords; i += 256) misc[i] = 0;
@@ -165,9 +165,8 @@ __device__ __forceinline__ bool tile_prefix(const uint32_t* st, int64_t tile, in
 // exclusive scans and plans the passes.  Clears the states of the first pass
 // that needs it and of the rank kernel.
 __global__ void __launch_bounds__(256)
-radix_hist_kernel(const uint64_t* __restrict__ key, uint32_t* __restrict__ misc,
-                  uint32_t* __restrict__ status, int64_t nstatus, uint32_t* __restrict__ tsum,
-                  int64_t ntsum, const Header* hdr)
+radix_hist_kernel(const uint64_t* key, uint32_t* misc, uint32_t* status, int64_t nstatus,
+                  uint32_t* tsum, int64_t ntsum, const Header* hdr)
 {
     __shared__ uint32_t cnt[8][256];
     __shared__ uint32_t wsum[8];
@@ -254,9 +253,8 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d)
 
 // One stable pass by the digit at 8 * pass (see the file's head).
 __global__ void __launch_bounds__(kSortThreads2, 2)
-radix_pass_kernel(uint64_t* __restrict__ key0, uint64_t* __restrict__ key1, uint32_t* __restrict__ pay0,
-                  uint32_t* __restrict__ pay1, uint32_t* __restrict__ status,
-                  uint32_t* __restrict__ misc, int pass, int wide, Header* hdr)
+radix_pass_kernel(uint64_t* key0, uint64_t* key1, uint32_t* pay0, uint32_t* pay1,
+                  uint32_t* status, uint32_t* misc, int pass, int wide, Header* hdr)
 {
     extern __shared__ __align__(16) unsigned char rsm[];
     uint64_t* skey = reinterpret_cast<uint64_t*>(rsm);
@@ -371,9 +369,8 @@ radix_pass_kernel(uint64_t* __restrict__ key0, uint64_t* __restrict__ key1, uint
 // written into the rank field of the packed element its payload names
 // (bit 31 selects the set: 0 = set0, 1 = set1).
 __global__ void __launch_bounds__(kSortThreads2)
-rank_write_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict__ key1,
-                  const uint32_t* __restrict__ pay0, const uint32_t* __restrict__ pay1,
-                  uint32_t* __restrict__ tsum, uint32_t* __restrict__ misc, KElem* pack0, KElem* pack1,
+rank_write_kernel(const uint64_t* key0, const uint64_t* key1, const uint32_t* pay0,
+                  const uint32_t* pay1, uint32_t* tsum, uint32_t* misc, KElem* pack0, KElem* pack1,
                   Header* hdr)
 {
     __shared__ uint32_t wcount[kSortWarps];
@@ -440,10 +437,9 @@ rank_write_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict_
 // Keys of the integration bounds a and b (one thread): 2 * (distinct ends
 // below q) + 1, or + 2 when q is itself an interval end; b = inf maps to the
 // rank of the last intervals.  Written to hdr->bound_key[0..1].
-__global__ void bound_keys_kernel(const uint64_t* __restrict__ key0, const uint64_t* __restrict__ key1,
-                                  const uint32_t* __restrict__ pay0, const uint32_t* __restrict__ pay1,
-                                  const uint32_t* __restrict__ misc, const KElem* pack0, const KElem* pack1, double a, double b,
-                                  Header* hdr)
+__global__ void bound_keys_kernel(const uint64_t* key0, const uint64_t* key1, const uint32_t* pay0,
+                                  const uint32_t* pay1, const uint32_t* misc, const KElem* pack0,
+                                  const KElem* pack1, double a, double b, Header* hdr)
 {
     chain_start();
     const int64_t m = (int64_t)hdr->nkeys;

@@ -54,11 +54,10 @@ __device__ __forceinline__ bool below_f32(double x)
 // for gaps below 2^-30 of their time.  Values outside the range of the float64
 // walks' integer products are noted in Header::wild.
 template <typename T, bool AUTO64>
-__global__ void validate_kernel(const int64_t* __restrict__ offsets,
-                                const T* __restrict__ times, const T* __restrict__ values,
+__global__ void validate_kernel(const int64_t* offsets, const T* times, const T* values,
                                 int64_t n, int64_t nnz_total, int whole, int walk_f32,
-                                int32_t* __restrict__ lens, uint32_t* __restrict__ skey,
-                                Header* hdr, int slot, int skip_on_error, int fs)
+                                int32_t* lens, uint32_t* skey, Header* hdr, int slot,
+                                int skip_on_error, int fs)
 {
     chain_start();
     // a collection built by an earlier kernel of the call is only checked
@@ -92,15 +91,11 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
             skey[i] = (tl > 0.f && tl < INFINITY) ? __float_as_uint(tl) : 0u;
         }
         local_max = max(local_max, (unsigned int)(o1 - o0));
-#pragma unroll 2
-        for (int64_t k = o0 + lane + 32 * part; k < o1; k += (int64_t)32 << fs) {
-            const T t = times[k];
-            const T v = values[k];
-            const T tp = k > o0 ? times[k - 1] : T(0);
+        auto check = [&](int64_t k, T t, T tp, T v) {
             // (every finite float32 suits)
             if constexpr (sizeof(T) == 8) wild |= !f64i_value_suits((uint64_t)__double_as_longlong(v));
-            if (!finite_val(t)) { record_error(hdr, kErrTimeNaN, k); continue; }
-            if (!finite_val(v)) { record_error(hdr, kErrValueNaN, k); continue; }
+            if (!finite_val(t)) { record_error(hdr, kErrTimeNaN, k); return; }
+            if (!finite_val(v)) { record_error(hdr, kErrValueNaN, k); return; }
             if (k == o0) {
                 if (!is_zero(t)) record_error(hdr, kErrT0, k);
             } else {
@@ -118,6 +113,16 @@ __global__ void validate_kernel(const int64_t* __restrict__ offsets,
                     record_error(hdr, kErrRange32, k);
                 }
             }
+        };
+        // two breakpoints' loads in flight per lane (the checks may record an
+        // error, which no coherent load is moved across)
+        const int64_t step = (int64_t)32 << fs;
+        for (int64_t k = o0 + lane + 32 * part; k < o1; k += 2 * step) {
+            const int64_t k2 = k + step < o1 ? k + step : k;
+            const T t = times[k], tp = k > o0 ? times[k - 1] : T(0), v = values[k];
+            const T t2 = times[k2], tp2 = k2 > o0 ? times[k2 - 1] : T(0), v2 = values[k2];
+            check(k, t, tp, v);
+            if (k2 != k) check(k2, t2, tp2, v2);
         }
     }
     if (__any_sync(0xffffffffu, need64) && lane == 0) atomicOr(&hdr->need64, 1u << slot);
@@ -145,10 +150,10 @@ __device__ __forceinline__ uint32_t length_bucket(int32_t len)
 }
 
 __global__ void __launch_bounds__(kSortThreads)
-sort_scan_kernel(const int32_t* __restrict__ lens, const uint32_t* __restrict__ skey, int64_t n,
+sort_scan_kernel(const int32_t* lens, const uint32_t* skey, int64_t n,
                  Header* hdr, int slot, int32_t* perm, int32_t* slen, uint32_t* khi0,
                  uint32_t* klo0, int32_t* kv0, uint32_t* khi1, uint32_t* klo1, int32_t* kv1,
-                 int64_t* __restrict__ poff)
+                 int64_t* poff)
 {
     __shared__ unsigned int hist[256];
     __shared__ unsigned int base[256];
@@ -290,9 +295,8 @@ sort_scan_kernel(const int32_t* __restrict__ lens, const uint32_t* __restrict__ 
 constexpr int kSortSmall = 1024;
 
 __global__ void __launch_bounds__(kSortSmall)
-sort_small_kernel(const int32_t* __restrict__ lens, const uint32_t* __restrict__ skey, int n,
-                  const Header* hdr, int slot, int32_t* __restrict__ perm, int32_t* __restrict__ slen,
-                  int64_t* __restrict__ poff)
+sort_small_kernel(const int32_t* lens, const uint32_t* skey, int n, const Header* hdr, int slot,
+                  int32_t* perm, int32_t* slen, int64_t* poff)
 {
     __shared__ unsigned long long xk[kSortSmall];
     __shared__ int32_t xi[kSortSmall];
@@ -356,11 +360,10 @@ template <> struct Elem<double, double> { using type = double2; };
 
 // 2^fs warps per sorted PCF: write its interval elements in the walk type.
 template <typename Tin, typename Tw>
-__global__ void pack_kernel(const int64_t* __restrict__ offsets, const Tin* __restrict__ times,
-                            const Tin* __restrict__ values, int64_t n,
-                            const int32_t* __restrict__ perm, const int32_t* __restrict__ slen,
-                            const int64_t* __restrict__ poff, void* packed_v, const Header* hdr,
-                            const unsigned int* gate, int want64, int fs)
+__global__ void pack_kernel(const int64_t* offsets, const Tin* times, const Tin* values, int64_t n,
+                            const int32_t* perm, const int32_t* slen, const int64_t* poff,
+                            void* packed_v, const Header* hdr, const unsigned int* gate, int want64,
+                            int fs)
 {
     using E = typename Elem<Tin, Tw>::type;
     chain_start();
@@ -376,11 +379,17 @@ __global__ void pack_kernel(const int64_t* __restrict__ offsets, const Tin* __re
         const int64_t o = offsets[src];
         const int64_t len = slen[s];
         const int64_t dst = poff[s];
-        for (int64_t k = lane + 32 * part; k < len; k += (int64_t)32 << fs) {
-            E e;
+        // two breakpoints' loads before the first store
+        const int64_t step = (int64_t)32 << fs;
+        for (int64_t k = lane + 32 * part; k < len; k += 2 * step) {
+            const int64_t k2 = k + step < len ? k + step : k;
+            E e, e2;
             e.x = (k + 1 < len) ? (Tw)times[o + k + 1] : (Tw)INFINITY;
             e.y = (Tw)values[o + k];
+            e2.x = (k2 + 1 < len) ? (Tw)times[o + k2 + 1] : (Tw)INFINITY;
+            e2.y = (Tw)values[o + k2];
             packed[dst + k] = e;
+            packed[dst + k2] = e2;
         }
     }
 }
@@ -394,11 +403,9 @@ __global__ void pack_kernel(const int64_t* __restrict__ offsets, const Tin* __re
 // float32 collection walked against a float64 one is packed the same way
 // (its times are exact in float64: lo = 0).
 template <typename Tin>
-__global__ void pack_keyed_kernel(const int64_t* __restrict__ offsets,
-                                  const Tin* __restrict__ times, const Tin* __restrict__ values,
-                                  int64_t n, const int32_t* __restrict__ perm,
-                                  const int32_t* __restrict__ slen, const int64_t* __restrict__ poff,
-                                  KElem* __restrict__ packed, KeyOut ko, const Header* hdr,
+__global__ void pack_keyed_kernel(const int64_t* offsets, const Tin* times, const Tin* values,
+                                  int64_t n, const int32_t* perm, const int32_t* slen,
+                                  const int64_t* poff, KElem* packed, KeyOut ko, const Header* hdr,
                                   const unsigned int* gate, int want64, int fs)
 {
     chain_start();
@@ -414,11 +421,10 @@ __global__ void pack_keyed_kernel(const int64_t* __restrict__ offsets,
         const int64_t o = offsets[src];
         const int64_t len = slen[s];
         const int64_t dst = poff[s];
-        for (int64_t k = lane + 32 * part; k < len; k += (int64_t)32 << fs) {
+        auto put = [&](int64_t k, double te, float v) {
             KElem e;
-            e.v = (float)values[o + k];
+            e.v = v;
             if (k + 1 < len) {
-                const double te = (double)times[o + k + 1];
                 const float hi = __double2float_rn(te);
                 e.k = 0;
                 e.hi = hi;
@@ -432,6 +438,16 @@ __global__ void pack_keyed_kernel(const int64_t* __restrict__ offsets,
                 e.lo = 0.f;
             }
             packed[dst + k] = e;
+        };
+        // two breakpoints' loads before the first store
+        const int64_t step = (int64_t)32 << fs;
+        for (int64_t k = lane + 32 * part; k < len; k += 2 * step) {
+            const int64_t k2 = k + step < len ? k + step : k;
+            const double te = k + 1 < len ? (double)times[o + k + 1] : 0.0;
+            const double te2 = k2 + 1 < len ? (double)times[o + k2 + 1] : 0.0;
+            const float v = (float)values[o + k], v2 = (float)values[o + k2];
+            put(k, te, v);
+            if (k2 != k) put(k2, te2, v2);
         }
     }
 }

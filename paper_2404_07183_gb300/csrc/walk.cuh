@@ -405,14 +405,16 @@ __device__ __forceinline__ double weight_span(double l, double dt, double lam, d
     else return exp(-lam * l) * (-expm1(-lam * dt)) * inv_lam;
 }
 
-// One 32-byte sector of global memory (32-byte aligned, read-only for the
-// kernel's lifetime) in a single 256-bit load.
+// One 32-byte sector of global memory (32-byte aligned) in a single 256-bit
+// load: coherent, and kept behind the kernel's wait, because the kernels that
+// write the packed elements may still run when this one starts.
 __device__ __forceinline__ void ldg_sector(const void* p, float (&r)[8])
 {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]),
-          "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
-        : "l"(p));
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]),
+                   "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+                 : "l"(p)
+                 : "memory");
 }
 
 __device__ __forceinline__ void decode_tile(const WalkArgs& a, int64_t t, int64_t& bi, int64_t& bj)
