@@ -539,6 +539,23 @@ int pcf_reduce_counters(const void* workspace, cudaStream_t stream, int64_t* pos
 int pcf_selftest_wait_timeout(int64_t polls, void* workspace, size_t workspace_bytes,
                               cudaStream_t stream);
 
+/*
+ * Self-test of the key sort's waits (float32 walks of float64 input; no
+ * counterpart in the paper).  Sorts and ranks `keys` (1 .. 2^24) keys
+ * (i + 1) * 0x9e3779b97f4a7c15 mod 2^64 >> 1 with at most `polls` (1 .. 2^20)
+ * polls per wait.  missing_pass -1: the whole sort; 0 .. 7: the first tile of
+ * that radix pass is never taken, 8: that of the rank kernel (more than 8,192
+ * keys, else PCF_EINVAL), so that the
+ * waits of its successors run out: nothing after that pass may write, and
+ * pcf_check(workspace) returns PCF_ETIMEOUT with reason 9.  *used: bytes of
+ * the workspace the call touches (set before PCF_ENOWS is returned for a
+ * smaller or NULL workspace); its last align256(16 * keys) bytes are 16-byte
+ * elements whose first 4 bytes are the ranks, 2 * (keys up to and including
+ * this one), or 0 when the ranks were not reached.
+ */
+int pcf_selftest_sort_wait(int64_t keys, int missing_pass, int64_t polls, void* workspace,
+                           size_t workspace_bytes, size_t* used, cudaStream_t stream);
+
 /* Bytes of the fixed device scratch array behind pcf_pairwise_noalloc. */
 #define PCF_NOALLOC_SCRATCH_BYTES (16u << 20)
 

@@ -43,6 +43,7 @@ SYMBOLS = ("pcf_workspace_size", "pcf_prepare", "pcf_pairwise", "pcf_cross", "pc
            "pcf_pairwise_ex", "pcf_cross_ex", "pcf_sort_order", "pcf_segment_integrals",
            "pcf_reduce_workspace_size", "pcf_reduce", "pcf_combine_workspace_size",
            "pcf_combine", "pcf_reduce_counters", "pcf_selftest_wait_timeout",
+           "pcf_selftest_sort_wait",
            "pcf_pairwise_backward_ex", "pcf_pairwise_to_host")
 PCF_RED_SUM, PCF_RED_MEAN, PCF_RED_MAX, PCF_RED_MIN, PCF_RED_STD = range(5)
 PCF_OP_ADD, PCF_OP_SUB, PCF_OP_MUL, PCF_OP_MAX, PCF_OP_MIN, PCF_OP_SQDIFF = range(6)
@@ -159,6 +160,8 @@ def load(build_if_missing: bool = False):
         lib.pcf_reduce_counters.argtypes = [P, P, ctypes.POINTER(I64), ctypes.POINTER(I64)]
         lib.pcf_selftest_wait_timeout.restype = I
         lib.pcf_selftest_wait_timeout.argtypes = [I64, P, SZ, P]
+        lib.pcf_selftest_sort_wait.restype = I
+        lib.pcf_selftest_sort_wait.argtypes = [I64, I, I64, P, SZ, ctypes.POINTER(SZ), P]
         lib.pcf_version.restype = ctypes.c_char_p
         lib.pcf_version.argtypes = []
         _lib = lib

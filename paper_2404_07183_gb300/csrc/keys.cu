@@ -18,13 +18,19 @@
 // patterns read as unsigned 64-bit integers.  One kernel counts all eight
 // 8-bit digits (they do not depend on the order) and plans the passes: a digit
 // that all keys share needs none.  Each pass is one kernel: a CTA takes a tile
-// of 8,192 keys by ticket, ranks them stably (warp match, per-warp digit
+// of 8,192 keys by ticket, ranks them stably (warp ballots, per-warp digit
 // counts), learns how many of each digit the tiles before it hold by decoupled
 // look-back (thread d waits for digit d; tickets make every predecessor a
 // running or finished CTA, and every wait is bounded), orders the tile in
 // shared memory and writes it in runs of one digit.  A last kernel counts
 // distinct keys the same way and writes every key's rank into the packed
 // element its payload names.
+//
+// A wait that gives up records kErrWait and leaves its tile unwritten.  From
+// then on no kernel may trust the buffers (a pass would scatter stale keys by
+// digit counts that are not theirs, the rank kernel would store through stale
+// payloads): every CTA of the passes, of the rank kernel and of the bounds
+// reads the recorded error first and returns.
 //
 // What bounds it: few keys, the latency of ten launches in a row; many, the
 // 24 bytes per key and pass.  A histogram, two scans and an unordered scatter
@@ -132,10 +138,21 @@ constexpr int64_t kNarrowKeys = 1ll << 27;
 // Polls before a look-back wait gives up (64 ns sleeps: 0.27 s and more).
 constexpr int kSortPolls = 1 << 22;
 
+// A CTA's tile of a pass (one thread): the next ticket, or -1 (stop) when an
+// error is recorded.
+__device__ __forceinline__ int64_t take_tile(uint32_t* ticket, const Header* hdr)
+{
+    const unsigned long long err = __ldcg(&hdr->err);
+    const int64_t t = (int64_t)atomicAdd(ticket, 1u);
+    return err == kNoError ? t : -1;
+}
+
 // Sum of the counts of the tiles before `tile` (stride words apart), by one
-// thread.  False when a wait gave up.
+// thread.  False when a wait gave up (after max_polls polls, or because
+// another one has).
 __device__ __forceinline__ bool tile_prefix(const uint32_t* st, int64_t tile, int stride,
-                                            const TileState& ts, const Header* hdr, uint32_t& prefix)
+                                            const TileState& ts, const Header* hdr, int max_polls,
+                                            uint32_t& prefix)
 {
     constexpr int kAhead = 8;               // states read at a time: one L2 latency for eight
     uint32_t sum = 0;
@@ -148,7 +165,7 @@ __device__ __forceinline__ bool tile_prefix(const uint32_t* st, int64_t tile, in
             const int64_t t = t0 - q;
             if (t < 0) break;                // (tile 0 publishes an inclusive prefix at once)
             for (int polls = 0; ts.empty(w[q]); ++polls) {
-                if (polls > kSortPolls || ((polls & 1023) == 1023 && __ldcg(&hdr->err) != kNoError))
+                if (polls > max_polls || ((polls & 1023) == 1023 && __ldcg(&hdr->err) != kNoError))
                     return false;
                 if (polls > 8) __nanosleep(64);
                 w[q] = __ldcg(st + t * stride);
@@ -254,7 +271,8 @@ __device__ __forceinline__ unsigned digit_peers(unsigned d)
 // One stable pass by the digit at 8 * pass (see the file's head).
 __global__ void __launch_bounds__(kSortThreads2, 2)
 radix_pass_kernel(uint64_t* key0, uint64_t* key1, uint32_t* pay0, uint32_t* pay1,
-                  uint32_t* status, uint32_t* misc, int pass, int wide, Header* hdr)
+                  uint32_t* status, uint32_t* misc, int pass, int wide, int max_polls,
+                  Header* hdr)
 {
     extern __shared__ __align__(16) unsigned char rsm[];
     uint64_t* skey = reinterpret_cast<uint64_t*>(rsm);
@@ -275,14 +293,14 @@ radix_pass_kernel(uint64_t* key0, uint64_t* key1, uint32_t* pay0, uint32_t* pay1
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const TileState ts{(uint32_t)pass + 1u, wide};
     if (tid == 0) {
-        s_tile = (int64_t)atomicAdd(&misc[kMiscTicket + pass], 1u);
+        s_tile = take_tile(&misc[kMiscTicket + pass], hdr);
         s_fail = 0;
     }
     for (int i = tid; i < kSortWarps * 256 / 2; i += kSortThreads2) reinterpret_cast<uint32_t*>(wcnt)[i] = 0;
     __syncthreads();
     const int64_t tile = s_tile, m = (int64_t)hdr->nkeys;
     const int64_t base = tile * kSortTile;
-    if (base >= m) return;                                  // nor any tile after it
+    if (tile < 0 || base >= m) return;                      // block-uniform (nor any tile after it)
     const int cnt = m - base < kSortTile ? (int)(m - base) : kSortTile;
     const int shift = 8 * pass;
     // warp w holds the tile's keys w * 512 .., item j of lane l is key 32 j + l
@@ -328,7 +346,7 @@ radix_pass_kernel(uint64_t* key0, uint64_t* key1, uint32_t* pay0, uint32_t* pay1
         dstart[tid] = incl - total;                         // within the warp, for now
         uint32_t prefix = 0;
         if (tile > 0) {
-            if (tile_prefix(st, tile, 256, ts, hdr, prefix))
+            if (tile_prefix(st, tile, 256, ts, hdr, max_polls, prefix))
                 atomicExch(st + tile * 256, ts.incl(prefix + real));
             else
                 s_fail = 1;
@@ -371,7 +389,7 @@ radix_pass_kernel(uint64_t* key0, uint64_t* key1, uint32_t* pay0, uint32_t* pay1
 __global__ void __launch_bounds__(kSortThreads2)
 rank_write_kernel(const uint64_t* key0, const uint64_t* key1, const uint32_t* pay0,
                   const uint32_t* pay1, uint32_t* tsum, uint32_t* misc, KElem* pack0, KElem* pack1,
-                  Header* hdr)
+                  int max_polls, Header* hdr)
 {
     __shared__ uint32_t wcount[kSortWarps];
     __shared__ uint32_t s_prefix;
@@ -383,13 +401,13 @@ rank_write_kernel(const uint64_t* key0, const uint64_t* key1, const uint32_t* pa
     const uint64_t* key = one ? key1 : key0;
     const uint32_t* pay = one ? pay1 : pay0;
     if (tid == 0) {
-        s_tile = (int64_t)atomicAdd(&misc[kMiscTicket + 8], 1u);
+        s_tile = take_tile(&misc[kMiscTicket + 8], hdr);
         s_fail = 0;
     }
     __syncthreads();
     const int64_t tile = s_tile, m = (int64_t)hdr->nkeys;
     const int64_t base = tile * kSortTile;
-    if (base >= m) return;
+    if (tile < 0 || base >= m) return;
     const int64_t w0 = base + warp * 32 * kSortItems;       // the warp's keys, in order
     uint32_t heads[kSortItems];                             // ballots: key differs from the one before
     uint32_t count = 0;
@@ -410,7 +428,7 @@ rank_write_kernel(const uint64_t* key0, const uint64_t* key1, const uint32_t* pa
         for (int w = 0; w < kSortWarps; ++w) { const uint32_t c = wcount[w]; wcount[w] = total; total += c; }
         atomicExch(tsum + tile, tile == 0 ? ts.incl(total) : ts.own(total));
         if (tile > 0) {
-            if (tile_prefix(tsum, tile, 1, ts, hdr, prefix)) atomicExch(tsum + tile, ts.incl(prefix + total));
+            if (tile_prefix(tsum, tile, 1, ts, hdr, max_polls, prefix)) atomicExch(tsum + tile, ts.incl(prefix + total));
             else s_fail = 1;
         }
         s_prefix = prefix;
@@ -442,6 +460,7 @@ __global__ void bound_keys_kernel(const uint64_t* key0, const uint64_t* key1, co
                                   const KElem* pack1, double a, double b, Header* hdr)
 {
     chain_start();
+    if (hdr->err != kNoError) return;       // the payloads may not be the sort's
     const int64_t m = (int64_t)hdr->nkeys;
     const uint64_t* key = misc[kMiscFinal] ? key1 : key0;
     const uint32_t* pay = misc[kMiscFinal] ? pay1 : pay0;
@@ -464,10 +483,11 @@ __global__ void bound_keys_kernel(const uint64_t* key0, const uint64_t* key1, co
     }
 }
 
-cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int64_t n0,
-                      KElem* pack1, const int64_t* poff1, int64_t n1, Header* hdr, cudaStream_t s)
+// The sort and the ranks, from the keys of ks.key[0], ks.pay[0] (hdr->nkeys of
+// them) and cleared counters.
+static cudaError_t sort_and_rank(const KeySort& ks, KElem* pack0, KElem* pack1, int max_polls,
+                                 Header* hdr, cudaStream_t s)
 {
-    launch_next(count_keys_kernel, 1, 256, 0, s, hdr, poff0, n0, poff1, n1, ks.misc);
     const unsigned tiles = (unsigned)ks.tiles;
     const int wide = ks.cap >= kNarrowKeys ? 1 : 0;
     cudaError_t e = cudaFuncSetAttribute(radix_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -486,11 +506,18 @@ cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int
             if (e != cudaSuccess) return e;
         }
         launch_next(radix_pass_kernel, tiles, kSortThreads2, radix_pass_smem(), s,
-            ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.status, ks.misc, pass, wide, hdr);
+            ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.status, ks.misc, pass, wide, max_polls, hdr);
     }
     launch_next(rank_write_kernel, tiles, kSortThreads2, 0, s, ks.key[0], ks.key[1], ks.pay[0], ks.pay[1], ks.tsum,
-                                                      ks.misc, pack0, pack1, hdr);
+                                                      ks.misc, pack0, pack1, max_polls, hdr);
     return cudaGetLastError();
+}
+
+cudaError_t rank_keys(const KeySort& ks, KElem* pack0, const int64_t* poff0, int64_t n0,
+                      KElem* pack1, const int64_t* poff1, int64_t n1, Header* hdr, cudaStream_t s)
+{
+    launch_next(count_keys_kernel, 1, 256, 0, s, hdr, poff0, n0, poff1, n1, ks.misc);
+    return sort_and_rank(ks, pack0, pack1, kSortPolls, hdr, s);
 }
 
 cudaError_t bound_keys(const KeySort& ks, const KElem* pack0, const KElem* pack1, double a, double b,
@@ -500,4 +527,48 @@ cudaError_t bound_keys(const KeySort& ks, const KElem* pack0, const KElem* pack1
     return cudaGetLastError();
 }
 
+// Self-test input: well mixed 63-bit keys, their own positions as payloads,
+// ranks zero; with missing >= 0, tile 0 of that pass is never handed out.
+__global__ void __launch_bounds__(256) sort_selftest_kernel(Header* hdr, uint64_t* key, uint32_t* pay,
+                                                            KElem* pack, int64_t keys, uint32_t* misc,
+                                                            int missing)
+{
+    const int64_t gid = (int64_t)blockIdx.x * 256 + threadIdx.x, gsz = (int64_t)gridDim.x * 256;
+    for (int64_t i = gid; i < keys; i += gsz) {
+        key[i] = ((uint64_t)(i + 1) * 0x9e3779b97f4a7c15ull) >> 1;
+        pay[i] = (uint32_t)i;
+        pack[i] = KElem{0u, 0.f, 0.f, 0.f};
+    }
+    for (int64_t i = gid; i < kMiscWords; i += gsz)
+        misc[i] = missing >= 0 && i == kMiscTicket + missing ? 1u : 0u;
+    if (gid == 0) {
+        hdr->err = kNoError;
+        hdr->nkeys = (unsigned long long)keys;
+    }
+}
+
 }  // namespace pcfgb
+
+extern "C" int pcf_selftest_sort_wait(int64_t keys, int missing_pass, int64_t polls, void* workspace,
+                                      size_t workspace_bytes, size_t* used, cudaStream_t stream)
+{
+    using namespace pcfgb;
+    if (keys < 1 || keys > (1ll << 24) || missing_pass < -1 || missing_pass > 8 || polls < 1 ||
+        polls > (1ll << 20) || !used)
+        return PCF_EINVAL;
+    // (with one tile there is no successor to wait for the missing one)
+    if (missing_pass >= 0 && keys <= kSortTile) return PCF_EINVAL;
+    *used = align_up(sizeof(Header)) + keysort_bytes(keys) + align_up(sizeof(KElem) * (size_t)keys);
+    if (!workspace || ((uintptr_t)workspace % kAlign) || workspace_bytes < *used) return PCF_ENOWS;
+    Header* hdr = (Header*)workspace;
+    char* cur = (char*)workspace + align_up(sizeof(Header));
+    const KeySort ks = carve_keysort(cur, keys);
+    KElem* pack = (KElem*)cur;
+    int64_t grid = (keys + 255) / 256;
+    if (grid > device_sm_count() * 8) grid = device_sm_count() * 8;
+    sort_selftest_kernel<<<(unsigned)grid, 256, 0, stream>>>(hdr, ks.key[0], ks.pay[0], pack, keys,
+                                                             ks.misc, missing_pass);
+    if (cudaGetLastError() != cudaSuccess) return PCF_ECUDA;
+    return sort_and_rank(ks, pack, nullptr, (int)polls, hdr, stream) == cudaSuccess ? PCF_OK
+                                                                                     : PCF_ECUDA;
+}
