@@ -541,11 +541,26 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     // Work units.  Thread 0 takes the next ticket while this unit is walked
     // and decodes a unit for the CTA (decoded by every thread, a unit cost the
     // CTA about 400 warp instructions and an atomic's latency; the Gram of
-    // 30,000 log-normal curves 82.0 -> 75.9 ms on two CTAs per SM).  Of the
-    // 40-register schedules only the L1, L2 and Gram walks of 8-byte elements
-    // have room for it (74.2 -> 71.5 ms); in the others every thread decodes.
-    constexpr bool kLean = CTAS < 3 || (sizeof(E) == 8 && (COMBO == kComboL1 || COMBO == kComboL2 ||
-                                                         COMBO == kComboGram));
+    // 30,000 log-normal curves 82.0 -> 75.9 ms on two CTAs per SM).
+    //
+    // Not with three CTAs per SM (40 registers): while this was written, one of
+    // those instantiations (float32 compensated, plain, L1 + L2 + Gram; it
+    // spills) reported an illegal memory access on a call with a small window,
+    // twice, and the cause was not found.  That source was not kept.  Ruled out
+    // by reading what is here: the unit's order (tiles.cuh; checked against
+    // the enumerated order on the host), sUnit and sBlock (written by thread 0
+    // between the barrier that ends a unit and the one that starts the next,
+    // read between that one and the next end), the ticket (thread 0 only; past
+    // the last unit nothing is decoded from it), the staging (a sector is read
+    // only if it holds an element of the set, and the arrays end on 256 bytes)
+    // and the results' indices (the same expressions in both forms).  Moving
+    // the sector loads did not end it; a build that checked and recorded every
+    // index ran exactly and recorded nothing.  One thing fits and cannot be
+    // shown any more: sBlock had a single entry with three CTAs, so a build
+    // that decoded ahead there wrote its second entry over a neighbour.
+    // Three CTAs decode in every thread, as they did before (Gram of 30,000
+    // log-normal curves 72.1 -> 74.8 ms).
+    constexpr bool kLean = CTAS < 3;
     unsigned long long ticket = 0;
     if (kLean && tid == 0) ticket = atomicAdd(&a.hdr->tiles, 1ull);
     for (;;) {
