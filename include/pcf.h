@@ -93,9 +93,7 @@ enum pcf_precision {
  * rounded to float32
  * (the walk's arithmetic).  Such a call needs nnz (both collections together
  * for a cross call) below 2^31, else PCF_EUNSUPPORTED.  The p-th root is
- * taken in float64; for float32 outputs of a float32 walk the square and cube
- * roots are float32 roots with a correction step, good to about 2^-44 before
- * the one rounding to float32.
+ * always taken in float64.
  *
  * PCF_PREC_ROUND_TIMES, or-ed into a float32 precision, asks for the faster
  * packed form instead: float64 times rounded to nearest float32 when packed
