@@ -163,7 +163,10 @@ enum pcf_cross_flags {
  *                         45,000 for float64), else TILE_512X3 for float32
  *                         walks of float32 input with one metric but general
  *                         p, TILE_512X2 for the others, TILE_1024 for
- *                         lambda > 0.  With rounded times or an explicit
+ *                         lambda > 0.  With more pairs but fewer tiles than
+ *                         half the SMs the longest PCF decides on the device
+ *                         between the tiles (even lengths) and the merge
+ *                         path.  With rounded times or an explicit
  *                         window: merge path when there are fewer tiles than
  *                         half the SMs, else TILE_1024 */
 enum pcf_sched_kernel {

@@ -436,29 +436,69 @@ int auto_tile_kernel(const pcf_integral* F, int nF, int form, bool weighted)
     return PCF_SCHED_TILE_512X3;
 }
 
-// Pairs up to which PCF_SCHED_AUTO takes the merge path.  It works in
-// proportion to the pairs, while a tile walk of few tiles takes one unit's
-// time however few pairs there are.  Measured (ms, tiles / merge path):
-// float32 walks, 5,050 pairs of 2 x 450 points 0.076 / 0.058 and of 2 x 900
-// 0.111 / 0.060, 20,100 pairs of 2 x 1,350 0.160 / 0.233 and of 2 x 275 (three
-// metrics) 0.109 / 0.100; float64 walks, 20,100 pairs of 2 x 55 points 0.109 /
-// 0.058 and of 2 x 275 (three metrics) 1.10 / 0.22, 45,150 pairs of 2 x 55
-// 0.109 / 0.100 and of 2 x 540 0.62 / 0.68.
+// What PCF_SCHED_AUTO launches: the tile walk for calls whose longest pair has at
+// most `even` advances and the merge path for the others (0: merge path only,
+// kAnySteps: tiles only).
+struct Route {
+    int tile;
+    int64_t even;
+};
+
+// Pairs up to which PCF_SCHED_AUTO takes the merge path whatever the lengths.  It
+// works in proportion to all advances, while a tile walk of few tiles takes its
+// longest pair's time however few pairs there are.  Walks alone (us, tiles /
+// merge path): float32, 5,050 pairs of 2 x 275 points 31 / 17, 12,880 of 2 x
+// 1,350 136 / 83; float64, 24,310 pairs of 2 x 55 points 47 / 46, 44,850 of 2 x
+// 275 208 / 181 and of 2 x 1,350 963 / 697.
 constexpr int64_t kMpPairsF32 = 14000, kMpPairsF64 = 45000;
 
-int auto_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool round,
-                bool windowed, bool weighted, const pcf_schedule* sched)
+// Beyond them, where there are fewer tiles than half the SMs (one unit per SM at
+// most), the longest pair decides: the tiles take longest * (a step of one
+// thread), the merge path pairs * mean * (an advance of the whole GPU), so tiles
+// when longest <= mean * pairs / K.  K from collections of 180 to 350 curves
+// (walks alone at 350, 61,425 pairs; us, tiles / merge path, one metric and three):
+// float32, 55 points 15 / 52 and 19 / 152, 275 33 / 83 and 43 / 161, 1,350 138 /
+// 318 and 183 / 370; float64 input in float32, 275 60 / 120 and 64 / 181, 1,350
+// 248 / 429 and 263 / 474; float64, 55 47 / 99 and 78 / 246, 275 208 / 253 and
+// 378 / 621, 1,350 965 / 976 and 1,786 / 2,273.  Uneven ones: float32, log-normal 138
+// / 66, with sigma 1.5 941 / 169, two of 50,000 points among short ones 3,317 /
+// 552; float64 log-normal 931 / 179.  Host rules see the mean only; the lengths are
+// known when the validation has run, so unless their bounds decide, both are
+// launched and one of them returns at once.  Whole calls, us, tiles only / this
+// rule / the walk of one warp per pair from before: 340 float32 curves, log-normal
+// 207 / 113 / 198, sigma 1.5 1,286 / 296 / 497, two of 50,000 points 3,396 / 675 /
+// 1,314; float64 1,110 / 254 / 321, 8,844 / 720 / 910, 20,994 / 896 / 1,913.
+int64_t even_limit(const WalkArgs& wa, int64_t pairs, int form, bool fused)
 {
+    const int64_t mean = wa.mean_steps;
+    // [form][mean > 700, > 256, shorter][one metric, fused]; short pairs leave the
+    // merge path its searches and combines
+    static const double k[3][3][2] = {{{50000, 50000}, {50000, 50000}, {25000, 15000}},     // float64
+                                      {{26000, 26000}, {22000, 14000}, {12000, 6000}},      // float32
+                                      {{34000, 34000}, {28000, 21000}, {20000, 7000}}};     // keyed
+    const double K = k[form][mean > 700 ? 0 : mean > 256 ? 1 : 2][fused ? 1 : 0];
+    const int64_t limit = (int64_t)((double)mean * (double)pairs / K);
+    if (limit >= wa.max_steps) return kAnySteps;
+    return limit < mean ? 0 : limit;
+}
+
+Route auto_route(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool round,
+                 bool windowed, bool weighted, const pcf_schedule* sched)
+{
+    const bool few_tiles = wa.ntiles * 2 < device_sm_count() && !windowed;
     // what a call with rounded times or an explicit window accepts depends on
     // the kernel (the merge path has no window to overflow): fewer tiles than
     // half the SMs go to the merge path there, as ever
     if (round || (sched && sched->window != 0))
-        return wa.ntiles * 2 < device_sm_count() && !windowed ? PCF_SCHED_MERGEPATH
-                                                              : PCF_SCHED_TILE_1024;
+        return {PCF_SCHED_TILE_1024, few_tiles ? 0 : kAnySteps};
+    const int tile = auto_tile_kernel(F, nF, form, weighted);
+    if (windowed) return {tile, kAnySteps};
     const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
-    if (!windowed && pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32))
-        return PCF_SCHED_MERGEPATH;
-    return auto_tile_kernel(F, nF, form, weighted);
+    if (pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32)) return {tile, 0};
+    if (!few_tiles) return {tile, kAnySteps};
+    bool fused = false;
+    for (const Launch& L : plan(F, nF)) fused = fused || L.n > 1;
+    return {tile, even_limit(wa, pairs, form, fused)};
 }
 
 bool is_windowed(const pcf_window* w)
@@ -494,19 +534,20 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
     const bool weighted = wa.lambda > 0.0;
     wa.shard_count = (sched && sched->shard_count > 1) ? sched->shard_count : 1;
     wa.shard_index = (sched && sched->shard_count > 1) ? sched->shard_index : 0;
-    int kernel = sched ? sched->kernel : PCF_SCHED_AUTO;
-    if (kernel == PCF_SCHED_AUTO)
-        kernel = auto_kernel(wa, F, nF, form, round, windowed, weighted, sched);
-    if (windowed && kernel == PCF_SCHED_MERGEPATH) return PCF_EUNSUPPORTED;
+    const int asked = sched ? sched->kernel : PCF_SCHED_AUTO;
+    const Route route = asked == PCF_SCHED_AUTO
+                            ? auto_route(wa, F, nF, form, round, windowed, weighted, sched)
+                            : Route{asked, asked == PCF_SCHED_MERGEPATH ? 0 : kAnySteps};
+    const int kernel = route.tile;
+    const bool tiles = route.even > 0, merge = route.even < kAnySteps;
+    if (windowed && merge) return PCF_EUNSUPPORTED;
     if (weighted && kernel != PCF_SCHED_TILE_1024) return PCF_EUNSUPPORTED;
-    if (kernel == PCF_SCHED_MERGEPATH && unit0 != 0) return PCF_EINVAL;
+    if (merge && unit0 != 0) return PCF_EINVAL;
 
     int64_t grid = 0;
     size_t smem = 0;
-    int64_t npairs = 0;
-    if (kernel == PCF_SCHED_MERGEPATH) {
-        npairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
-    } else {
+    const int64_t npairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
+    if (tiles) {
         const bool half = kernel == PCF_SCHED_TILE_512X2 || kernel == PCF_SCHED_TILE_512X3;
         const int ctas = kernel == PCF_SCHED_TILE_512X3 ? 3 : (half ? 2 : 1);
         const int regions = half ? 3 : 4;   // 32 x 16 or 32 x 32 units
@@ -537,10 +578,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
             wa.root[k] = f.apply_root ? 1 : 0;
             wa.p[k] = f.metric == PCF_LP ? f.p : (f.metric == PCF_L2 ? 2.0 : 1.0);
         }
-        if (kernel != PCF_SCHED_MERGEPATH)
-            launch_kernel(wa.at_once != 0, reset_tiles_kernel, 1, 1, 0, s, wa.hdr,
-                          (unsigned long long)unit0);
-        cudaError_t e;
+        cudaError_t e = cudaSuccess;
         const int g = (int)grid;
         // launcher of (schedule, precision, form)
 #define PCF_PICK(sfx)                                                                       \
@@ -548,20 +586,24 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
          : precision == PCF_PREC_F32_COMP ? (keyed ? launch_walk_f32ck_##sfx : launch_walk_f32c_##sfx) \
          : precision == PCF_PREC_F32_BLOCK ? (keyed ? launch_walk_f32bk_##sfx : launch_walk_f32b_##sfx) \
          : (keyed ? launch_walk_f32k_##sfx : launch_walk_f32_##sfx))
-        if (kernel == PCF_SCHED_MERGEPATH) {
+        if (tiles) {
+            wa.steps_lo = 0;
+            wa.steps_hi = route.even;
+            launch_kernel(wa.at_once != 0, reset_tiles_kernel, 1, 1, 0, s, wa.hdr,
+                          (unsigned long long)unit0);
+            if (kernel == PCF_SCHED_TILE_512X3) e = PCF_PICK(t512x3)(L.combo, wa, g, smem, s);
+            else if (kernel == PCF_SCHED_TILE_512X2) e = PCF_PICK(t512)(L.combo, wa, g, smem, s);
+            else if (weighted) e = PCF_PICK(t1024w)(L.combo, wa, g, smem, s);
+            else e = PCF_PICK(t1024)(L.combo, wa, g, smem, s);
+        }
+        if (merge && e == cudaSuccess) {
+            wa.steps_lo = route.even;
+            wa.steps_hi = kAnySteps;
             auto mp = precision == PCF_PREC_F64 ? launch_mergepath_f64
                     : precision == PCF_PREC_F32_COMP ? (keyed ? launch_mergepath_f32ck : launch_mergepath_f32c)
                     : precision == PCF_PREC_F32_BLOCK ? (keyed ? launch_mergepath_f32bk : launch_mergepath_f32b)
                     : (keyed ? launch_mergepath_f32k : launch_mergepath_f32);
-            e = mp(L.combo, wa, npairs, wa.mean_steps, s);
-        } else if (kernel == PCF_SCHED_TILE_512X3) {
-            e = PCF_PICK(t512x3)(L.combo, wa, g, smem, s);
-        } else if (kernel == PCF_SCHED_TILE_512X2) {
-            e = PCF_PICK(t512)(L.combo, wa, g, smem, s);
-        } else if (weighted) {
-            e = PCF_PICK(t1024w)(L.combo, wa, g, smem, s);
-        } else {
-            e = PCF_PICK(t1024)(L.combo, wa, g, smem, s);
+            e = mp(L.combo, wa, npairs, s);
         }
 #undef PCF_PICK
         if (e != cudaSuccess) return PCF_ECUDA;
@@ -782,6 +824,7 @@ int pcf_pairwise_ex(const pcf_csr* x, const pcf_integral* F, int nF, int precisi
     wa.n_r = wa.n_c = x->n;
     wa.nb_r = wa.nb_c = (x->n + kTile - 1) / kTile;
     wa.mean_steps = 2 * (x->nnz / x->n);
+    wa.max_steps = 2 * (x->nnz - x->n + 1);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;
@@ -852,6 +895,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     wa.n_r = wa.n_c = N;
     wa.nb_r = wa.nb_c = (N + kTile - 1) / kTile;
     wa.mean_steps = 2 * (x->nnz / N);
+    wa.max_steps = 2 * (x->nnz - N + 1);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;
@@ -913,8 +957,12 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     pcf_schedule sch;
     memset(&sch, 0, sizeof sch);
     if (schedule) sch = *schedule;
-    if (sch.kernel == PCF_SCHED_AUTO)
-        sch.kernel = auto_kernel(wa, F, nF, form, pr.round, false, false, schedule);
+    bool whole = sch.kernel == PCF_SCHED_MERGEPATH || nbands == 1;
+    if (sch.kernel == PCF_SCHED_AUTO) {
+        const Route route = auto_route(wa, F, nF, form, pr.round, false, false, schedule);
+        if (route.even < kAnySteps) whole = true;    // the merge path, or the choice, in one piece
+        else sch.kernel = route.tile;
+    }
     // `stream` continues after the last copy enqueued, also when a later
     // step fails (the caller may reuse the buffers after an error)
     auto join = [&]() -> bool {
@@ -928,7 +976,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     };
     auto fail = [&](int code) { join(); return code; };
     int64_t permuted = 0;   // sorted rows whose columns are back in the input order
-    if (sch.kernel == PCF_SCHED_MERGEPATH || nbands == 1) {
+    if (whole) {
         rc = run_walks_for(wa, F, nF, pr, form, &sch, nullptr, stream);
         if (rc != PCF_OK) return rc;
         if (!copy_rows(0, N)) return fail(PCF_ECUDA);
@@ -1064,6 +1112,7 @@ static int cross_impl(const pcf_csr* a, const pcf_csr* b, int64_t row_begin, int
     wa.nb_c = (b->n + kTile - 1) / kTile;
     wa.ntiles = wa.nb_r * wa.nb_c;
     wa.mean_steps = a->nnz / (a->n > 0 ? a->n : 1) + b->nnz / b->n;   // (a: of the whole set)
+    wa.max_steps = a->nnz - a->n + 1 + b->nnz - b->n + 1;
     wa.symmetric = 0;
     wa.hdr = hdr;
     wa.layout = PCF_OUT_FULL;
@@ -1335,6 +1384,7 @@ int pcf_pairwise_weighted(const pcf_csr* x, const pcf_csr* w, const pcf_integral
     wa.n_r = wa.n_c = m.n;
     wa.nb_r = wa.nb_c = (m.n + kTile - 1) / kTile;
     wa.mean_steps = 2 * (m.nnz / m.n);
+    wa.max_steps = 2 * (m.nnz - m.n + 1);
     wa.ntiles = wa.nb_r * (wa.nb_r + 1) / 2;
     wa.symmetric = 1;
     wa.hdr = hdr;

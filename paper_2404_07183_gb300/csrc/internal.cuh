@@ -236,6 +236,9 @@ struct WalkArgs {
     int64_t nb_r, nb_c;      // tile blocks
     int64_t ntiles;
     int64_t mean_steps;      // mean breakpoints of a pair (both PCFs), for the host's choices
+    int64_t max_steps;       // bound on a pair's advances, likewise
+    int64_t steps_lo, steps_hi;  // the launch walks when the longest pair of the call has
+                             // more than steps_lo and at most steps_hi advances
     int symmetric;           // pairwise: upper-triangle tiles, R == C
     int tile_order;          // symmetric tile order: 0 = column blocks from the last
                              // down, 1 = row blocks from the first up (each with its
@@ -264,7 +267,20 @@ struct WalkArgs {
     int gate_want64;             // (*gate != 0) == gate_want64; null = always runs
 };
 
+constexpr int64_t kAnySteps = INT64_MAX;   // WalkArgs::steps_hi: no bound
+
 #ifdef __CUDACC__
+// Device-side choice between the walks of a call by the lengths the validation
+// found: exactly one of the launches whose (steps_lo, steps_hi] cover all
+// lengths walks.  (A pair has n_f + n_g - 2 finite ends; 2 more are counted,
+// alike for all.)
+__device__ __forceinline__ bool steps_gated_off(const WalkArgs& a)
+{
+    if (a.steps_lo == 0 && a.steps_hi == kAnySteps) return false;
+    const int64_t longest = (int64_t)a.hdr->maxlen[0] + (int64_t)a.hdr->maxlen[a.symmetric ? 0 : 1];
+    return longest <= a.steps_lo || longest > a.steps_hi;
+}
+
 // Device-side choice between the float32 and float64 walks of an AUTO64 call.
 __device__ __forceinline__ bool gated_off(const unsigned int* gate, int want64)
 {
@@ -286,14 +302,13 @@ enum Combo : int {
 };
 
 // Launch the persistent tile walk for one precision, CTA size and metric
-// combination, or the cooperative merge-path walk over `npairs` pairs of
-// `mean_steps` breakpoints (both PCFs) on average.
+// combination, or the cooperative merge-path walk over `npairs` pairs.
 #define PCF_DECL_WALK(name)                                                                     \
     cudaError_t launch_walk_##name##_t1024(int, const WalkArgs&, int, size_t, cudaStream_t);    \
     cudaError_t launch_walk_##name##_t512(int, const WalkArgs&, int, size_t, cudaStream_t);     \
     cudaError_t launch_walk_##name##_t512x3(int, const WalkArgs&, int, size_t, cudaStream_t);   \
     cudaError_t launch_walk_##name##_t1024w(int, const WalkArgs&, int, size_t, cudaStream_t);   \
-    cudaError_t launch_mergepath_##name(int, const WalkArgs&, int64_t, int64_t, cudaStream_t);
+    cudaError_t launch_mergepath_##name(int, const WalkArgs&, int64_t, cudaStream_t);
 PCF_DECL_WALK(f64)
 PCF_DECL_WALK(f32c)
 PCF_DECL_WALK(f32)

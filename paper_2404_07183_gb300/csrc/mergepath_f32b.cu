@@ -2,8 +2,8 @@
 #include "mergepath.cuh"
 
 namespace pcfgb {
-cudaError_t launch_mergepath_f32b(int combo, const WalkArgs& a, int64_t npairs, int64_t mean_steps, cudaStream_t s)
+cudaError_t launch_mergepath_f32b(int combo, const WalkArgs& a, int64_t npairs, cudaStream_t s)
 {
-    return launch_mergepath_t<float, kF32B>(combo, a, npairs, mean_steps, s);
+    return launch_mergepath_t<float, kF32B>(combo, a, npairs, s);
 }
 }  // namespace pcfgb

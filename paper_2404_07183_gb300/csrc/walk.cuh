@@ -439,6 +439,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
 
     chain_wait();
     if (gated_off(a.gate, a.gate_want64)) return;   // the other walk of an AUTO64 call
+    if (steps_gated_off(a)) return;                 // the merge path walks
     if (block_sees_error(a.hdr)) return;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

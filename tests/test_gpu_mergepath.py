@@ -99,3 +99,55 @@ def test_auto_keeps_what_windows_and_rounding_accept(pcf):
     v = np.tile(np.concatenate([np.arange(t.size - 1) % 7, [0.0]]), 200)
     pcf.pcf_pairwise(pcf.PcfTensors.from_numpy(synth.PcfSet(o, np.tile(t, 200), v), "cuda"), ["l1"],
                      precision="f32c_round")
+
+
+@pytest.mark.parametrize("lens", [[40000, 33000, 20001], [2, 60000, 50000, 1]], ids=str)
+@pytest.mark.parametrize("prec,dtype", [("f64", np.float64), ("f32c", np.float64), ("f32c", np.float32)])
+def test_clusters_of_eight(pcf, lens, prec, dtype):
+    """Eight CTAs per pair, also where some of them get no advance, whole and in
+    shards."""
+    import torch
+    rng = np.random.default_rng(len(lens))
+    s = synth.from_lengths(lens, lambda r, m: r.exponential(1.0, m),
+                           lambda r, o: np.where(np.isin(np.arange(o[-1]), o[1:] - 1), 0.0,
+                                                 r.standard_normal(o[-1])), rng, dtype)
+    x = pcf.PcfTensors.from_numpy(s, "cuda")
+    s64 = synth.PcfSet(s.offsets, s.times.astype(np.float64), s.values.astype(np.float64))
+    diag = np.array([oracle.segment_sq(*s64.pcf(i)) for i in range(s64.n)])
+    metrics = ["l1", "l2", "gram"]
+    got = pcf.pcf_pairwise(x, metrics, precision=prec, out_dtype=torch.float64, schedule="mergepath")
+    parts = [torch.full_like(g, -7.0) for g in got]
+    for k in range(4):
+        pcf.pcf_pairwise(x, metrics, precision=prec, out=parts, schedule="mergepath", shard=(k, 4))
+    for m, g, p in zip(metrics, got, parts):
+        assert max_rel_error(m, g.cpu().numpy(), oracle.matrix(s64, metric=m), diag) <= TOL[prec], m
+        assert torch.equal(g, p), m
+
+
+@pytest.mark.parametrize("prec,dtype", [("f64", np.float64), ("f32c", np.float64), ("f32c", np.float32),
+                                        ("f32b", np.float32), ("f32", np.float32)])
+@pytest.mark.parametrize("kind", ["short", "edge of the copy", "one long", "many", "skewed"])
+def test_warps_and_ctas(pcf, kind, prec, dtype):
+    """A warp per pair around its copied length (256 advances) and for many pairs
+    of more than 1,024; one very long curve decides for CTAs on the device."""
+    import torch
+    rng = np.random.default_rng(21)
+    lens = {"short": rng.integers(1, 40, 60),
+            "edge of the copy": np.array([128, 129, 130, 131, 1, 2, 256, 257, 258, 127]),
+            "one long": np.concatenate([rng.integers(5, 30, 40), [5000]]),
+            "many": rng.integers(500, 800, 50),
+            "skewed": np.concatenate([rng.integers(100, 300, 78), [30000, 9000]])}[kind]
+    s = synth.from_lengths(lens, lambda r, m: r.exponential(1.0, m),
+                           lambda r, o: np.where(np.isin(np.arange(o[-1]), o[1:] - 1), 0.0,
+                                                 r.standard_normal(o[-1])), rng, dtype)
+    x = pcf.PcfTensors.from_numpy(s, "cuda")
+    s64 = synth.PcfSet(s.offsets, s.times.astype(np.float64), s.values.astype(np.float64))
+    diag = np.array([oracle.segment_sq(*s64.pcf(i)) for i in range(s64.n)])
+    tol = {**TOL, "f32": 5e-4}[prec]
+    for metrics in (["l1"], ["l1", "l2", "gram"], [("lp", 3.0)]):
+        got = pcf.pcf_pairwise(x, metrics, precision=prec, out_dtype=torch.float64,
+                               schedule="mergepath")
+        for m, g in zip(metrics, got):
+            code, p = (m, 1.0) if isinstance(m, str) else m
+            assert max_rel_error(code, g.cpu().numpy(), oracle.matrix(s64, metric=code, p=p),
+                                 diag) <= tol, m
