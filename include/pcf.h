@@ -162,8 +162,9 @@ enum pcf_cross_flags {
  *   PCF_SCHED_AUTO        merge path for few pairs (14,000 for float32 walks,
  *                         45,000 for float64), else TILE_512X3 for float32
  *                         walks of float32 input with one metric but general
- *                         p, TILE_512X2 for the others, TILE_1024 for
- *                         lambda > 0.  With more pairs but fewer tiles than
+ *                         p and more units than two per SM, TILE_512X2 for
+ *                         the others, TILE_1024 for lambda > 0.  With more
+ *                         pairs but fewer tiles than
  *                         half the SMs the longest PCF decides on the device
  *                         between the tiles (even lengths) and the merge
  *                         path.  With rounded times or an explicit

@@ -423,14 +423,16 @@ int check_window(const pcf_window* w)
 // 96.3 / 82.0 / 76.9; float32 cross 3,001 x 4,000 of 1,000 points with three
 // metrics 20.8 / 19.2 / 19.8; float64 N = 1,000 0.461 / 0.407 / 0.414.  Two
 // CTAs let one issue while the other waits at a tile barrier.  The third pays
-// where 40 registers hold the walk: 8-byte elements and one metric without
-// pow.  TILE_1024 stays for the exp(-lambda t) weights, which only it has, and
-// (auto_kernel) where its larger window decides what is accepted: rounded
-// times, whose coincident times must fit one window, and explicit windows.
-int auto_tile_kernel(const pcf_integral* F, int nF, int form, bool weighted)
+// where 40 registers hold the walk (8-byte elements and one metric without pow)
+// and two per SM do not hold all units: with fewer, some SMs get three CTAs and
+// others one (450 even curves of 1,350 points 291 or 384 us per call, 280 with
+// two per SM).  TILE_1024 stays for the exp(-lambda t) weights, which only it
+// has, and (auto_route) where its larger window decides what is accepted:
+// rounded times, whose coincident times must fit one window, and explicit windows.
+int auto_tile_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool weighted)
 {
     if (weighted) return PCF_SCHED_TILE_1024;
-    if (form != kPackF32) return PCF_SCHED_TILE_512X2;
+    if (form != kPackF32 || wa.ntiles <= device_sm_count()) return PCF_SCHED_TILE_512X2;
     for (const Launch& L : plan(F, nF))
         if (L.n > 1 || L.combo == kComboLP) return PCF_SCHED_TILE_512X2;
     return PCF_SCHED_TILE_512X3;
@@ -491,7 +493,7 @@ Route auto_route(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bo
     // half the SMs go to the merge path there, as ever
     if (round || (sched && sched->window != 0))
         return {PCF_SCHED_TILE_1024, few_tiles ? 0 : kAnySteps};
-    const int tile = auto_tile_kernel(F, nF, form, weighted);
+    const int tile = auto_tile_kernel(wa, F, nF, form, weighted);
     if (windowed) return {tile, kAnySteps};
     const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
     if (pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32)) return {tile, 0};
