@@ -570,6 +570,9 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
         const int64_t units = wa.ntiles * (half ? 2 : 1) - unit0;
         if (grid > units) grid = units;
         if (grid < 1) return PCF_OK;
+        // tickets of this shard (bands: from unit 0 on), but for the last 16 per CTA
+        wa.ahead_before = (wa.ntiles - wa.shard_index + wa.shard_count - 1) / wa.shard_count *
+                              (half ? 2 : 1) - 16 * grid;
     }
     for (const Launch& L : plan(F, nF)) {
         wa.nout = L.n;

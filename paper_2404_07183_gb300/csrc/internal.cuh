@@ -235,6 +235,7 @@ struct WalkArgs {
     int64_t n_r, n_c;
     int64_t nb_r, nb_c;      // tile blocks
     int64_t ntiles;
+    int64_t ahead_before;    // tickets below this one take the CTA's next one ahead
     int64_t mean_steps;      // mean breakpoints of a pair (both PCFs), for the host's choices
     int64_t max_steps;       // bound on a pair's advances, likewise
     int64_t steps_lo, steps_hi;  // the launch walks when the longest pair of the call has

@@ -500,7 +500,13 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     // Work units.  Thread 0 takes the next ticket while this unit is walked
     // and decodes a unit for the CTA (decoded by every thread, a unit cost the
     // CTA about 400 warp instructions and an atomic's latency; the Gram of
-    // 30,000 log-normal curves 82.0 -> 75.9 ms on two CTAs per SM).
+    // 30,000 log-normal curves 82.0 -> 75.9 ms on two CTAs per SM).  Not for
+    // the last 16 units per CTA: a ticket held while a long unit is walked keeps
+    // its unit from the CTAs that are done, up to 40% of a call of few units (700
+    // curves, exp(-lambda t) weights in float64: 20.8 ms with tickets always
+    // ahead, 15.9 so; L1 of 1,000 log-normal curves 1.98 ms, 1.28), while taking
+    // it late costs an atomic's latency per unit (float32 curves of 20 points, N =
+    // 6,000: 786 us always ahead, 791 so, 797 for the last 32, 830 never).
     //
     // Not with three CTAs per SM (40 registers): while this was written, one of
     // those instantiations (float32 compensated, plain, L1 + L2 + Gram; it
@@ -521,10 +527,11 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
     // log-normal curves 72.1 -> 74.8 ms).
     constexpr bool kLean = CTAS < 3;
     unsigned long long ticket = 0;
-    if (kLean && tid == 0) ticket = atomicAdd(&a.hdr->tiles, 1ull);
+    bool ahead = false;                             // (thread 0) the ticket is taken already
     for (;;) {
         if (tid == 0) {
-            const int64_t k = (int64_t)(kLean ? ticket : atomicAdd(&a.hdr->tiles, 1ull));
+            if (!kLean || !ahead) ticket = atomicAdd(&a.hdr->tiles, 1ull);
+            const int64_t k = (int64_t)ticket;
             const int64_t u = (a.shard_index + (k / UNITS) * a.shard_count) * UNITS + (k % UNITS);
             sUnit = u;
             if (kLean && u / UNITS < a.ntiles) {
@@ -532,7 +539,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) walk_kernel(const WalkArgs a)
                 decode_tile(a, u / UNITS, r, c);
                 sBlock[0] = r;
                 sBlock[1] = c;
-                ticket = atomicAdd(&a.hdr->tiles, 1ull);
+                ahead = k < a.ahead_before;
+                if (ahead) ticket = atomicAdd(&a.hdr->tiles, 1ull);
             }
         }
         __syncthreads();
