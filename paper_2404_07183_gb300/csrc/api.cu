@@ -440,11 +440,12 @@ int auto_tile_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form
 
 // What PCF_SCHED_AUTO launches: the tile walk for calls whose longest pair has at
 // most `even` advances and the merge path for the others (0: merge path only,
-// kAnySteps: tiles only).
+// kAnySteps: tiles only, kByLaunch: even_limit of each launch).
 struct Route {
     int tile;
     int64_t even;
 };
+constexpr int64_t kByLaunch = -1;
 
 // Pairs up to which PCF_SCHED_AUTO takes the merge path whatever the lengths.  It
 // works in proportion to all advances, while a tile walk of few tiles takes its
@@ -455,33 +456,43 @@ struct Route {
 constexpr int64_t kMpPairsF32 = 14000, kMpPairsF64 = 45000;
 
 // Beyond them, where there are fewer tiles than half the SMs (one unit per SM at
-// most), the longest pair decides: the tiles take longest * (a step of one
-// thread), the merge path pairs * mean * (an advance of the whole GPU), so tiles
-// when longest <= mean * pairs / K.  K from collections of 180 to 350 curves
-// (walks alone at 350, 61,425 pairs; us, tiles / merge path, one metric and three):
-// float32, 55 points 15 / 52 and 19 / 152, 275 33 / 83 and 43 / 161, 1,350 138 /
-// 318 and 183 / 370; float64 input in float32, 275 60 / 120 and 64 / 181, 1,350
-// 248 / 429 and 263 / 474; float64, 55 47 / 99 and 78 / 246, 275 208 / 253 and
-// 378 / 621, 1,350 965 / 976 and 1,786 / 2,273.  Uneven ones: float32, log-normal 138
-// / 66, with sigma 1.5 941 / 169, two of 50,000 points among short ones 3,317 /
-// 552; float64 log-normal 931 / 179.  Host rules see the mean only; the lengths are
-// known when the validation has run, so unless their bounds decide, both are
-// launched and one of them returns at once.  Whole calls, us, tiles only / this
-// rule / the walk of one warp per pair from before: 340 float32 curves, log-normal
-// 207 / 113 / 198, sigma 1.5 1,286 / 296 / 497, two of 50,000 points 3,396 / 675 /
-// 1,314; float64 1,110 / 254 / 321, 8,844 / 720 / 910, 20,994 / 896 / 1,913.
-int64_t even_limit(const WalkArgs& wa, int64_t pairs, int form, bool fused)
+// most), the longest pair decides: a tile walk takes t0 + t * longest (one thread
+// walks a pair), the merge path pairs * (p + c * mean).  The constants are fits to
+// even collections of 180 to 350 curves, walks alone; at 350 (61,425 pairs; us,
+// tiles / merge path, one metric and three): float32, 55 points 15 / 52 and 19 /
+// 152, 275 33 / 83 and 43 / 161, 1,350 138 / 318 and 183 / 370; float64 input in
+// float32, 55 19 / 56 and 21 / 154, 275 60 / 120 and 64 / 181, 1,350 248 / 429 and
+// 263 / 474; float64, 55 47 / 99 and 78 / 246, 275 208 / 253 and 378 / 621, 1,350
+// 965 / 976 and 1,786 / 2,273.  A root by pow, taken by one lane per pair on the
+// merge path, adds 5 ns to a pair, a square root 0.5.  Host rules see the mean only; the lengths are
+// known when the validation has run, so both are launched (where even lengths
+// gain more by the tiles than that costs) and one of them returns at once.  Whole
+// calls, us, tiles only / this rule / the former walk of one warp per pair: 340
+// float32 curves, log-normal 207 / 113 / 198, sigma 1.5 1,286 / 296 / 497, two of
+// 50,000 points 3,396 / 675 / 1,314; float64 1,110 / 254 / 321, 8,844 / 720 / 910,
+// 20,994 / 896 / 1,913.
+struct WalkCost { double p, c, t0, t; };   // us per pair, per advance; us, us per advance
+
+int64_t even_limit(const WalkArgs& wa, const Launch& L, const pcf_integral* F, int form)
 {
-    const int64_t mean = wa.mean_steps;
-    // [form][mean > 700, > 256, shorter][one metric, fused]; short pairs leave the
-    // merge path its searches and combines
-    static const double k[3][3][2] = {{{50000, 50000}, {50000, 50000}, {25000, 15000}},     // float64
-                                      {{26000, 26000}, {22000, 14000}, {12000, 6000}},      // float32
-                                      {{34000, 34000}, {28000, 21000}, {20000, 7000}}};     // keyed
-    const double K = k[form][mean > 700 ? 0 : mean > 256 ? 1 : 2][fused ? 1 : 0];
-    const int64_t limit = (int64_t)((double)mean * (double)pairs / K);
-    if (limit >= wa.max_steps) return kAnySteps;
-    return limit < mean ? 0 : limit;
+    // [form][one metric, three]
+    static const WalkCost costs[3][2] = {
+        {{0.9e-3, 5.6e-6, 10, 0.35}, {2.7e-3, 12.7e-6, 12, 0.655}},     // float64
+        {{0.6e-3, 1.8e-6, 9, 0.047}, {2.2e-3, 1.6e-6, 11, 0.064}},      // float32
+        {{0.6e-3, 2.5e-6, 10, 0.088}, {2.1e-3, 2.3e-6, 12, 0.093}}};    // keyed
+    constexpr double kSecondLaunch = 12;    // us
+    WalkCost w = costs[form][L.n > 1 ? 1 : 0];
+    if ((L.combo == kComboLP || L.combo == kComboL3 || L.combo == kComboL1L2L3) &&
+        F[L.idx[L.n - 1]].apply_root)
+        w.p += 5e-3;
+    else if (L.combo == kComboL2 && F[L.idx[0]].apply_root)
+        w.p += 0.5e-3;
+    const double pairs = wa.symmetric ? 0.5 * (double)wa.n_r * (double)(wa.n_r + 1)
+                                      : (double)wa.n_r * (double)wa.n_c;
+    const double mean = (double)wa.mean_steps, merge = pairs * (w.p + w.c * mean);
+    if (merge - (w.t0 + w.t * mean) < kSecondLaunch) return 0;
+    const double limit = (merge - w.t0) / w.t;
+    return limit >= (double)wa.max_steps ? kAnySteps : (int64_t)limit;
 }
 
 Route auto_route(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool round,
@@ -497,10 +508,7 @@ Route auto_route(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bo
     if (windowed) return {tile, kAnySteps};
     const int64_t pairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
     if (pairs <= (form == kPackF64 ? kMpPairsF64 : kMpPairsF32)) return {tile, 0};
-    if (!few_tiles) return {tile, kAnySteps};
-    bool fused = false;
-    for (const Launch& L : plan(F, nF)) fused = fused || L.n > 1;
-    return {tile, even_limit(wa, pairs, form, fused)};
+    return {tile, few_tiles ? kByLaunch : kAnySteps};
 }
 
 bool is_windowed(const pcf_window* w)
@@ -541,7 +549,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
                             ? auto_route(wa, F, nF, form, round, windowed, weighted, sched)
                             : Route{asked, asked == PCF_SCHED_MERGEPATH ? 0 : kAnySteps};
     const int kernel = route.tile;
-    const bool tiles = route.even > 0, merge = route.even < kAnySteps;
+    const bool tiles = route.even != 0, merge = route.even != kAnySteps;   // (at all)
     if (windowed && merge) return PCF_EUNSUPPORTED;
     if (weighted && kernel != PCF_SCHED_TILE_1024) return PCF_EUNSUPPORTED;
     if (merge && unit0 != 0) return PCF_EINVAL;
@@ -591,9 +599,10 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
          : precision == PCF_PREC_F32_COMP ? (keyed ? launch_walk_f32ck_##sfx : launch_walk_f32c_##sfx) \
          : precision == PCF_PREC_F32_BLOCK ? (keyed ? launch_walk_f32bk_##sfx : launch_walk_f32b_##sfx) \
          : (keyed ? launch_walk_f32k_##sfx : launch_walk_f32_##sfx))
-        if (tiles) {
+        const int64_t even = route.even == kByLaunch ? even_limit(wa, L, F, form) : route.even;
+        if (even > 0) {
             wa.steps_lo = 0;
-            wa.steps_hi = route.even;
+            wa.steps_hi = even;
             launch_kernel(wa.at_once != 0, reset_tiles_kernel, 1, 1, 0, s, wa.hdr,
                           (unsigned long long)unit0);
             if (kernel == PCF_SCHED_TILE_512X3) e = PCF_PICK(t512x3)(L.combo, wa, g, smem, s);
@@ -601,8 +610,8 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
             else if (weighted) e = PCF_PICK(t1024w)(L.combo, wa, g, smem, s);
             else e = PCF_PICK(t1024)(L.combo, wa, g, smem, s);
         }
-        if (merge && e == cudaSuccess) {
-            wa.steps_lo = route.even;
+        if (even < kAnySteps && e == cudaSuccess) {
+            wa.steps_lo = even;
             wa.steps_hi = kAnySteps;
             auto mp = precision == PCF_PREC_F64 ? launch_mergepath_f64
                     : precision == PCF_PREC_F32_COMP ? (keyed ? launch_mergepath_f32ck : launch_mergepath_f32c)
@@ -965,7 +974,7 @@ int pcf_pairwise_to_host(const pcf_csr* x, const pcf_integral* F, int nF, int pr
     bool whole = sch.kernel == PCF_SCHED_MERGEPATH || nbands == 1;
     if (sch.kernel == PCF_SCHED_AUTO) {
         const Route route = auto_route(wa, F, nF, form, pr.round, false, false, schedule);
-        if (route.even < kAnySteps) whole = true;    // the merge path, or the choice, in one piece
+        if (route.even != kAnySteps) whole = true;   // the merge path, or the choice, in one piece
         else sch.kernel = route.tile;
     }
     // `stream` continues after the last copy enqueued, also when a later
