@@ -554,8 +554,10 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
     if (weighted && kernel != PCF_SCHED_TILE_1024) return PCF_EUNSUPPORTED;
     if (merge && unit0 != 0) return PCF_EINVAL;
 
+    const int chained = wa.at_once;
     int64_t grid = 0;
     size_t smem = 0;
+    bool spread = false;
     const int64_t npairs = wa.symmetric ? wa.n_r * (wa.n_r + 1) / 2 : wa.n_r * wa.n_c;
     if (tiles) {
         const bool half = kernel == PCF_SCHED_TILE_512X2 || kernel == PCF_SCHED_TILE_512X3;
@@ -578,6 +580,12 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
         const int64_t units = wa.ntiles * (half ? 2 : 1) - unit0;
         if (grid > units) grid = units;
         if (grid < 1) return PCF_OK;
+        // As a dependent of the preparation's kernels, a grid smaller than the GPU
+        // is placed while those still hold some SMs, and ends up doubled on the
+        // others: float64, 64 x 1,100 curves of 50 to 500 points with three metrics
+        // (140 CTAs) 1.24 ms per call, 0.69 launched in the ordinary way, which
+        // costs a call about 4 us.  So it is, unless the walk is short.
+        spread = grid < (int64_t)sms * ctas && wa.mean_steps >= (form == kPackF64 ? 128 : 1024);
         // tickets of this shard (bands: from unit 0 on), but for the last 16 per CTA
         wa.ahead_before = (wa.ntiles - wa.shard_index + wa.shard_count - 1) / wa.shard_count *
                               (half ? 2 : 1) - 16 * grid;
@@ -603,8 +611,9 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
         if (even > 0) {
             wa.steps_lo = 0;
             wa.steps_hi = even;
-            launch_kernel(wa.at_once != 0, reset_tiles_kernel, 1, 1, 0, s, wa.hdr,
+            launch_kernel(chained != 0, reset_tiles_kernel, 1, 1, 0, s, wa.hdr,
                           (unsigned long long)unit0);
+            wa.at_once = chained && !spread ? 1 : 0;
             if (kernel == PCF_SCHED_TILE_512X3) e = PCF_PICK(t512x3)(L.combo, wa, g, smem, s);
             else if (kernel == PCF_SCHED_TILE_512X2) e = PCF_PICK(t512)(L.combo, wa, g, smem, s);
             else if (weighted) e = PCF_PICK(t1024w)(L.combo, wa, g, smem, s);
