@@ -543,7 +543,7 @@ int pcf_selftest_wait_timeout(int64_t polls, void* workspace, size_t workspace_b
 
 /*
  * Self-test of the key sort's waits (float32 walks of float64 input; no
- * counterpart in the paper).  Sorts and ranks `keys` (1 .. 2^24) keys
+ * counterpart in the paper).  Sorts and ranks `keys` (1 .. 2^28) keys
  * (i + 1) * 0x9e3779b97f4a7c15 mod 2^64 >> 1 with at most `polls` (1 .. 2^20)
  * polls per wait.  missing_pass -1: the whole sort; 0 .. 7: the first tile of
  * that radix pass is never taken, 8: that of the rank kernel (more than 8,192

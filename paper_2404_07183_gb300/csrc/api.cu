@@ -583,7 +583,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
         // As a dependent of the preparation's kernels, a grid smaller than the GPU
         // is placed while those still hold some SMs, and ends up doubled on the
         // others: float64, 64 x 1,100 curves of 50 to 500 points with three metrics
-        // (140 CTAs) 1.24 ms per call, 0.69 launched in the ordinary way, which
+        // (140 CTAs) 1.28 ms per call, 0.75 launched in the ordinary way, which
         // costs a call about 4 us.  So it is, unless the walk is short.
         spread = grid < (int64_t)sms * ctas && wa.mean_steps >= (form == kPackF64 ? 128 : 1024);
         // tickets of this shard (bands: from unit 0 on), but for the last 16 per CTA

@@ -35,8 +35,8 @@
 // What bounds it: few keys, the latency of ten launches in a row; many, the
 // 24 bytes per key and pass.  A histogram, two scans and an unordered scatter
 // per pass (35 launches) came before: three matrices of 701 stable-rank curves
-// (193,000 keys) took 0.78 ms per call and now 0.47, of 20,000 (5.5 million)
-// 117.0 and now 116.2.
+// (193,000 keys) took 0.78 ms per call and 0.47 with this sort, of 20,000 (5.5
+// million) 117.0 and 116.2.
 //
 // The number of keys is known on the device only (it depends on the lengths
 // of the rows a call packs); the kernels read it from the header and are
@@ -553,7 +553,7 @@ extern "C" int pcf_selftest_sort_wait(int64_t keys, int missing_pass, int64_t po
                                       size_t workspace_bytes, size_t* used, cudaStream_t stream)
 {
     using namespace pcfgb;
-    if (keys < 1 || keys > (1ll << 24) || missing_pass < -1 || missing_pass > 8 || polls < 1 ||
+    if (keys < 1 || keys > (1ll << 28) || missing_pass < -1 || missing_pass > 8 || polls < 1 ||
         polls > (1ll << 20) || !used)
         return PCF_EINVAL;
     // (with one tile there is no successor to wait for the missing one)

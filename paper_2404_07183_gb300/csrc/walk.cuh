@@ -5,8 +5,9 @@
 //   * PCFs are sorted by length and cut into blocks of 32; a tile is a
 //     (row block, column block) pair: 32 x 32 = 1024 pairs.  Pairwise calls
 //     visit the upper triangle of blocks; cross calls all blocks.  Tiles are
-//     handed out by one atomic counter (longest PCFs first) to one persistent
-//     1024-thread CTA per SM.
+//     handed out by one atomic counter (longest PCFs first) to persistent
+//     CTAs: one of 1,024 threads per SM, or two or three of 512, which take
+//     half tiles of 32 x 16 pairs.
 //   * Warp w of the CTA takes the tile's w-th diagonal: lane l walks the pair
 //     (row (l + w) mod 32, column l).  Every lane of a half-warp (quarter-warp
 //     for 16-byte elements) therefore reads a different PCF of each side.

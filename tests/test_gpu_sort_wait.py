@@ -54,6 +54,25 @@ def test_whole_sort(pcf, keys):
     assert not ranks[:, 1:].any()
 
 
+@pytest.mark.parametrize("missing", [-1, 3])
+def test_wide_states(pcf, missing):
+    """2^27 keys and more: states without a pass number, cleared before each pass."""
+    import torch
+    from paper_2404_07183_gb300 import abi
+    keys = (1 << 27) + 5
+    status, _, ranks, intact = _run(pcf, keys, missing, 1 << 20 if missing < 0 else 500)
+    assert intact
+    if missing >= 0:
+        assert status == abi.PCF_ETIMEOUT and not ranks.any()
+        return
+    i = torch.arange(1, keys + 1, dtype=torch.int64, device="cuda")
+    key = (i * -7046029254386353131 >> 1) & 0x7FFFFFFFFFFFFFFF     # 0x9e3779b97f4a7c15
+    place = torch.empty_like(i)
+    place[torch.argsort(key)] = torch.arange(keys, dtype=torch.int64, device="cuda")
+    got = torch.from_numpy(np.ascontiguousarray(ranks[:, 0]).astype(np.int64))
+    assert status == 0 and torch.equal(got, 2 * (place.cpu() + 1))
+
+
 @pytest.mark.parametrize("missing", range(9))
 @pytest.mark.parametrize("keys", [8193, 70001, 3000000])
 def test_a_wait_that_gives_up_stops_the_sort(pcf, keys, missing):
