@@ -161,15 +161,15 @@ enum pcf_cross_flags {
  *                         (for few pairs)
  *   PCF_SCHED_AUTO        merge path for few pairs (14,000 for float32 walks,
  *                         45,000 for float64), else TILE_512X3 for float32
- *                         walks of float32 input with one metric but general
- *                         p and more units than two per SM, TILE_512X2 for
- *                         the others, TILE_1024 for lambda > 0.  With more
- *                         pairs but fewer tiles than
- *                         half the SMs the longest PCF decides on the device
- *                         between the tiles (even lengths) and the merge
- *                         path.  With rounded times or an explicit
- *                         window: merge path when there are fewer tiles than
- *                         half the SMs, else TILE_1024 */
+ *                         walks of float32 input with one of L1, L2 and Gram,
+ *                         up to 120 breakpoints on average and more units
+ *                         than two per SM, TILE_512X2 for the others,
+ *                         TILE_1024 for lambda > 0.  With more pairs but
+ *                         fewer tiles than half the SMs the longest PCF
+ *                         decides on the device between the tiles (even
+ *                         lengths) and the merge path.  With rounded times
+ *                         or an explicit window: merge path when there are
+ *                         fewer tiles than half the SMs, else TILE_1024 */
 enum pcf_sched_kernel {
     PCF_SCHED_AUTO = 0, PCF_SCHED_TILE_1024 = 1, PCF_SCHED_TILE_512X2 = 2,
     PCF_SCHED_MERGEPATH = 3, PCF_SCHED_TILE_512X3 = 4

@@ -420,21 +420,28 @@ int check_window(const pcf_window* w)
 // 1024-thread CTA per SM / two / three 512-thread CTAs): stable-rank curves
 // N = 6,000, float64 input in float32 with one metric 9.99 / 9.42 / 9.52, with
 // three 11.57 / 10.62 / 11.00; float32 Gram of 30,000 log-normal curves
-// 96.3 / 82.0 / 76.9; float32 cross 3,001 x 4,000 of 1,000 points with three
-// metrics 20.8 / 19.2 / 19.8; float64 N = 1,000 0.461 / 0.407 / 0.414.  Two
-// CTAs let one issue while the other waits at a tile barrier.  The third pays
-// where 40 registers hold the walk (8-byte elements and one metric without pow)
-// and two per SM do not hold all units: with fewer, some SMs get three CTAs and
-// others one (450 even curves of 1,350 points 291 or 384 us per call, 280 with
-// two per SM).  TILE_1024 stays for the exp(-lambda t) weights, which only it
-// has, and (auto_route) where its larger window decides what is accepted:
-// rounded times, whose coincident times must fit one window, and explicit windows.
+// 78.4 / 72.6 / 73.5, L1 of 20,000 stable-rank ones 56.4 / 53.8 / 55.3; float32
+// cross 3,001 x 4,000 of 1,000 points with three metrics 20.8 / 19.2 / 19.8; float64
+// N = 1,000 0.461 / 0.407 / 0.414.  Two CTAs let one issue while the other waits at
+// a tile barrier.  The third pays where 40 registers hold the walk (8-byte elements,
+// L1, L2 or Gram alone) and pairs are short, so that barriers come often: float32 L1
+// of 1,500 curves of 55 points 0.122 / 0.104 / 0.102, of 3,000 of 20 0.268 / 0.219 /
+// 0.206, but of 1,000 of 275 0.192 / 0.178 / 0.190; and where two per SM do not hold
+// all units: with fewer, some SMs get three CTAs and others one (450 even curves
+// of 1,350 points 291 or 384 us per call, 280 with two per SM).  TILE_1024 stays
+// for the exp(-lambda t) weights, which only it has, and (auto_route) where its
+// larger window decides what is accepted: rounded times, whose coincident times
+// must fit one window, and explicit windows.
+constexpr int64_t kThreeCtaSteps = 240;
+
 int auto_tile_kernel(const WalkArgs& wa, const pcf_integral* F, int nF, int form, bool weighted)
 {
     if (weighted) return PCF_SCHED_TILE_1024;
-    if (form != kPackF32 || wa.ntiles <= device_sm_count()) return PCF_SCHED_TILE_512X2;
+    if (form != kPackF32 || wa.ntiles <= device_sm_count() || wa.mean_steps > kThreeCtaSteps)
+        return PCF_SCHED_TILE_512X2;
     for (const Launch& L : plan(F, nF))
-        if (L.n > 1 || L.combo == kComboLP) return PCF_SCHED_TILE_512X2;
+        if (L.combo != kComboL1 && L.combo != kComboL2 && L.combo != kComboGram)
+            return PCF_SCHED_TILE_512X2;
     return PCF_SCHED_TILE_512X3;
 }
 
@@ -464,13 +471,13 @@ constexpr int64_t kMpPairsF32 = 14000, kMpPairsF64 = 45000;
 // float32, 55 19 / 56 and 21 / 154, 275 60 / 120 and 64 / 181, 1,350 248 / 429 and
 // 263 / 474; float64, 55 47 / 99 and 78 / 246, 275 208 / 253 and 378 / 621, 1,350
 // 965 / 976 and 1,786 / 2,273.  A root by pow, taken by one lane per pair on the
-// merge path, adds 5 ns to a pair, a square root 0.5.  Host rules see the mean only; the lengths are
-// known when the validation has run, so both are launched (where even lengths
-// gain more by the tiles than that costs) and one of them returns at once.  Whole
-// calls, us, tiles only / this rule / the former walk of one warp per pair: 340
-// float32 curves, log-normal 207 / 113 / 198, sigma 1.5 1,286 / 296 / 497, two of
-// 50,000 points 3,396 / 675 / 1,314; float64 1,110 / 254 / 321, 8,844 / 720 / 910,
-// 20,994 / 896 / 1,913.
+// merge path, adds 5 ns to a pair, a square root 0.5.  Host rules see the mean
+// only; the lengths are known when the validation has run, so both are launched
+// (where even lengths gain more by the tiles than that costs) and one of them
+// returns at once.  Whole calls, us, tiles only / this rule / the former walk of
+// one warp per pair: 340 float32 curves, log-normal 207 / 113 / 198, sigma 1.5
+// 1,286 / 296 / 497, two of 50,000 points 3,396 / 675 / 1,314; float64 1,110 / 254
+// / 321, 8,844 / 720 / 910, 20,994 / 896 / 1,913.
 struct WalkCost { double p, c, t0, t; };   // us per pair, per advance; us, us per advance
 
 int64_t even_limit(const WalkArgs& wa, const Launch& L, const pcf_integral* F, int form)
@@ -618,6 +625,7 @@ int run_walks(WalkArgs& wa, const pcf_integral* F, int nF, int precision, int fo
             else if (kernel == PCF_SCHED_TILE_512X2) e = PCF_PICK(t512)(L.combo, wa, g, smem, s);
             else if (weighted) e = PCF_PICK(t1024w)(L.combo, wa, g, smem, s);
             else e = PCF_PICK(t1024)(L.combo, wa, g, smem, s);
+            wa.at_once = chained;
         }
         if (even < kAnySteps && e == cudaSuccess) {
             wa.steps_lo = even;
