@@ -74,14 +74,14 @@ def fp64_ops(metrics, schedule):
 # DRAM bytes (read + write) per launch of the benchmark's compensated walk,
 # from one ncu capture (profiles/walk_f32ck_dram_traffic_stable_rank_n20000.md),
 # valid only while the walk's source is the one that was measured.
-TRAFFIC_RECORD = {"source_sha256_16": "edd8e1ec5b550ed1+4091e163e9ee196c",
-                  "by_schedule_layout": {("tile512x2", "full"): 1192259584 + 4747656192}}
+TRAFFIC_RECORD = {"source_sha256_16": "cc2725023c6ebcce+f841d3bb7b6f3402+91c300a6c9e926ed",
+                  "by_schedule_layout": {("tile512x2", "full"): 1196367616 + 4748920832}}
 
 
 def walk_source_id():
     import hashlib
     parts = []
-    for f in ("walk.cuh", "internal.cuh"):
+    for f in ("walk.cuh", "internal.cuh", "tiles.cuh"):
         with open(os.path.join(ROOT, "paper_2404_07183_gb300", "csrc", f), "rb") as fh:
             parts.append(hashlib.sha256(fh.read()).hexdigest()[:16])
     return "+".join(parts)
