@@ -113,3 +113,19 @@ def test_a_replay_chooses_again(pcf):
         want = pcf.pcf_pairwise(y, ["l1"], precision="f32c", out_dtype=torch.float64)[0]
         assert torch.equal(got, want)
         assert max_rel_error("l1", got.cpu().numpy(), oracle.matrix(s, metric="l1")) <= 1e-5
+
+
+@pytest.mark.parametrize("long", [0, 9000])
+def test_promoted_and_weighted_calls(pcf, long):
+    """AUTO64 where the float64 walk runs, and a weight PCF."""
+    import torch
+    s = _set(330, long, np.float64)
+    big = synth.PcfSet(s.offsets, s.times, s.values * 1e60)
+    x, y = pcf.PcfTensors.from_numpy(s, "cuda"), pcf.PcfTensors.from_numpy(big, "cuda")
+    want = pcf.pcf_pairwise(y, ["l1"], precision="f64", out_dtype=torch.float64)[0]
+    got = pcf.pcf_pairwise(y, ["l1"], precision="f32c_auto64", out_dtype=torch.float64)[0]
+    assert torch.equal(got, want)
+    one = (np.array([0.0]), np.array([1.0]))
+    plain = pcf.pcf_pairwise(x, ["l1"], precision="f64", out_dtype=torch.float64)[0]
+    weighted = pcf.pcf_pairwise_weighted(x, one, ["l1"], precision="f64", out_dtype=torch.float64)[0]
+    torch.testing.assert_close(weighted, plain, rtol=1e-12, atol=0.0)
