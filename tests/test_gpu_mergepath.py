@@ -1,6 +1,7 @@
 """The cooperative merge path at the edges of its slabs, groups and parts
-(needs a GPU).  A warp takes 256 advances per slab, a CTA 2,048; a pair goes to
-CTAs above 1,024 breakpoints on average and to clusters of 2, 4 or 8 CTAs above
+(needs a GPU).  A warp copies float64 pairs of up to 256 advances, a CTA takes
+2,048 per slab; above 1,024 breakpoints per pair on average a long longest pair
+sends the call to CTAs, and few long pairs to clusters of 2, 4 or 8 of them above
 8,192, 16,384 and 32,768."""
 import numpy as np
 import pytest
